@@ -1,4 +1,5 @@
-// msp_fft.cuh -- shared-memory-resident 2-D FFT building blocks for sm_103a.
+// msp_fft.cuh -- 2-D FFT building blocks for sm_103a: line transforms by thread groups (W = 64, 256), small
+// transforms in registers (W = 128), and the residual of the far field.
 //
 // The Fourier operator F of the multislice model (Sec. 2.1 / 2.2) is the
 // unnormalised 2-D DFT of a W x W wave.  A W-point line transform is split
@@ -212,6 +213,210 @@ __device__ __forceinline__ void line_fft(float2 (&v)[W / T], const Tw& tw, float
 #pragma unroll
     for (int k2 = 0; k2 < T; ++k2) v[mc + NC * k2] = INV ? cconj(X[k2]) : X[k2];
   }
+}
+
+// ---------------------------------------------------------------------------
+// residual of the far field
+// ---------------------------------------------------------------------------
+// Amplitude-flow residual of a far-field value: the factor f of R = f Psi, f = 1 - sqrt(I) / |Psi| (1 where
+// Psi counts as zero), and the loss term added to `lsum`.
+__device__ __forceinline__ float residual_exact(float a2, float I, float zthr2, float& lsum) {
+  const float a = sqrtf(a2), rt = sqrtf(I);
+  const float d = rt - a;
+  lsum = fmaf(d, d, lsum);
+  return (a2 > zthr2) ? (1.f - rt / a) : 1.f;   // a2 > zthr2 >= 0 implies a > 0
+}
+// The same for finite a2 and finite I >= 0 without a branch: zero counts are the usual case in a pattern, and
+// the library's square root and quotient leave their short path for zero operands (measured: of 165
+// thousand cycles per position, W = 128, L = 4, 19 went into this pass; W = 64, L = 5, 2115 positions,
+// loss and gradients: 398 -> 383 us).  sqrt(x) = s + (x - s s) y / 2 and n / a = q + (n - q a) y from the
+// reciprocal square root y, with one fused residual each (Markstein 1990).
+__device__ __forceinline__ float residual_finite(float a2, float I, float zthr2, float& lsum) {
+  const float y = rsqrtf(a2), z = rsqrtf(I);
+  float a = a2 * y, rt = I * z;
+  a = fmaf(fmaf(-a, a, a2), 0.5f * y, a);
+  rt = fmaf(fmaf(-rt, rt, I), 0.5f * z, rt);
+  a = a2 > 0.f ? a : 0.f;
+  rt = I > 0.f ? rt : 0.f;
+  const float d = rt - a;
+  lsum = fmaf(d, d, lsum);
+  float q = rt * y;
+  q = fmaf(fmaf(-q, a, rt), y, q);
+  return a2 > zthr2 ? 1.f - q : 1.f;
+}
+__device__ __forceinline__ bool residual_is_finite(float a2, float I) {
+  return a2 <= 3.402823466e+38f && I >= 0.f && I <= 3.402823466e+38f;
+}
+
+// v <- f v for N far-field values of a thread and their measured intensities.
+template <int N>
+__device__ __forceinline__ void residual(float2 (&v)[N], const float (&I)[N], float zthr2, float& lsum) {
+  bool finite = true;
+#pragma unroll
+  for (int m = 0; m < N; ++m) finite = finite && residual_is_finite(fmaf(v[m].x, v[m].x, v[m].y * v[m].y), I[m]);
+#pragma unroll
+  for (int m = 0; m < N; ++m) {
+    const float a2 = fmaf(v[m].x, v[m].x, v[m].y * v[m].y);
+    const float f = finite ? residual_finite(a2, I[m], zthr2, lsum) : residual_exact(a2, I[m], zthr2, lsum);
+    v[m] = make_float2(v[m].x * f, v[m].y * f);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// small DFTs in registers, both directions
+// ---------------------------------------------------------------------------
+// cos(2 pi k / 32) for k = 0..8 (the regular 32-gon), sin by symmetry
+__host__ __device__ constexpr double cos32(int k) {
+  constexpr double c[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
+                           0.70710678118654752440, 0.55557023301960222474, 0.38268343236508977173,
+                           0.19509032201612826785, 0.0};
+  return k <= 8 ? c[k] : -c[16 - k];
+}
+__host__ __device__ constexpr double sin32(int k) { return k <= 8 ? cos32(8 - k) : cos32(k - 8); }
+
+// Packed FP32 pairs (sm_100 and later): one instruction works on both components.  The FP32 pipe runs
+// them at half the rate of the scalar instructions (measured: 1.87 against 3.72 warp instructions per
+// clock and SM), so they halve the issue slots and leave the arithmetic rate as it is.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {   // a b + c
+  float2 d;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
+      "fma.rn.f32x2 x, x, y, z;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+#define MSP_PACKED_OP(name, op)                                                                            \
+  __device__ __forceinline__ float2 name(float2 a, float2 b) {                                             \
+    float2 d;                                                                                              \
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t" op " x, x, y;\n\t"      \
+        "mov.b64 {%0, %1}, x;\n\t}"                                                                        \
+        : "=f"(d.x), "=f"(d.y)                                                                             \
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));                                                         \
+    return d;                                                                                              \
+  }
+MSP_PACKED_OP(add2, "add.rn.f32x2")
+MSP_PACKED_OP(sub2, "sub.rn.f32x2")
+MSP_PACKED_OP(mul2, "mul.rn.f32x2")
+#undef MSP_PACKED_OP
+
+// Two complex values side by side, (re0, re1) and (im0, im1).
+struct C2 {
+  float2 re, im;
+};
+__device__ __forceinline__ C2 add(C2 a, C2 b) { return {add2(a.re, b.re), add2(a.im, b.im)}; }
+__device__ __forceinline__ C2 sub(C2 a, C2 b) { return {sub2(a.re, b.re), sub2(a.im, b.im)}; }
+__device__ __forceinline__ float2 add(float2 a, float2 b) { return cadd(a, b); }
+__device__ __forceinline__ float2 sub(float2 a, float2 b) { return csub(a, b); }
+// e + i o, e - i o
+__device__ __forceinline__ void quarter(C2 e, C2 o, C2& p, C2& m) {
+  p = {sub2(e.re, o.im), add2(e.im, o.re)};
+  m = {add2(e.re, o.im), sub2(e.im, o.re)};
+}
+__device__ __forceinline__ void quarter(float2 e, float2 o, float2& p, float2& m) {
+  p = make_float2(e.x - o.y, e.y + o.x);
+  m = make_float2(e.x + o.y, e.y - o.x);
+}
+// u = (re + q im, im - q re)
+__device__ __forceinline__ C2 rot_tan(C2 o, float q) {
+  const float2 p = make_float2(q, q), n = make_float2(-q, -q);
+  return {fma2(p, o.im, o.re), fma2(n, o.re, o.im)};
+}
+__device__ __forceinline__ float2 rot_tan(float2 o, float q) {
+  return make_float2(fmaf(q, o.y, o.x), fmaf(-q, o.x, o.y));
+}
+// u = (q re + im, q im - re)
+__device__ __forceinline__ C2 rot_cot(C2 o, float q) {
+  const float2 p = make_float2(q, q), one = make_float2(-1.f, -1.f);
+  return {fma2(p, o.re, o.im), fma2(p, o.im, mul2(one, o.re))};
+}
+__device__ __forceinline__ float2 rot_cot(float2 o, float q) {
+  return make_float2(fmaf(q, o.x, o.y), fmaf(q, o.y, -o.x));
+}
+__device__ __forceinline__ C2 axpy(float m, C2 u, C2 e) {   // m u + e
+  const float2 p = make_float2(m, m);
+  return {fma2(p, u.re, e.re), fma2(p, u.im, e.im)};
+}
+__device__ __forceinline__ float2 axpy(float m, float2 u, float2 e) {
+  return make_float2(fmaf(m, u.x, e.x), fmaf(m, u.y, e.y));
+}
+
+// The butterfly e + w o, e - w o with w = exp(-2 pi i K / N) (INV: conjugated), 0 <= K < N / 2, on one
+// complex value (float2) or two (C2).  w is applied as its larger component times (1, tan) or (cot, 1),
+// |tan|, |cot| <= 1: two fused multiply-adds for the rotation and four that scale and add, six
+// operations where a complex product and two sums take eight, with no more roundings on the way.
+template <int N, int K, bool INV, typename T>
+__device__ __forceinline__ void butterfly(T e, T o, T& x0, T& x1) {
+  if constexpr (K == 0) {
+    x0 = add(e, o);
+    x1 = sub(e, o);
+  } else if constexpr (4 * K == N) {   // w = -i (INV: +i)
+    if constexpr (INV) quarter(e, o, x0, x1);
+    else quarter(e, o, x1, x0);
+  } else {
+    constexpr int k = K * (32 / N);
+    constexpr double c = cos32(k), s = INV ? -sin32(k) : sin32(k);   // w o = (c re + s im, c im - s re)
+    if constexpr (c * c >= s * s) {
+      const T u = rot_tan(o, (float)(s / c));
+      x0 = axpy((float)c, u, e);
+      x1 = axpy((float)-c, u, e);
+    } else {
+      const T u = rot_cot(o, (float)(c / s));
+      x0 = axpy((float)s, u, e);
+      x1 = axpy((float)-s, u, e);
+    }
+  }
+}
+template <int N, int K, bool INV, typename T>
+__device__ __forceinline__ void butterflies(const T* E, const T* O, T* X) {
+  if constexpr (K < N / 2) {
+    butterfly<N, K, INV>(E[K], O[K], X[K], X[K + N / 2]);
+    butterflies<N, K + 1, INV>(E, O, X);
+  }
+}
+// X[k] = sum_n x[n S] exp(-+2 pi i n k / N), N <= 32 (radix-2 decimation in time, unrolled)
+template <int N, int S, bool INV, typename T>
+__device__ __forceinline__ void fft(const T* x, T* X) {
+  if constexpr (N == 1) {
+    X[0] = x[0];
+  } else {
+    T E[N / 2], O[N / 2];
+    fft<N / 2, 2 * S, INV>(x, E);
+    fft<N / 2, 2 * S, INV>(x + S, O);
+    butterflies<N, 0, INV>(E, O, X);
+  }
+}
+
+// A 32-point transform as two 16-point ones side by side in pairs and one stage of scalars.
+// fft32_dif: scalars in, spectrum out in pairs (X[2i], X[2i+1]); ifft32_dit: pairs in, scalars out.
+template <int K>
+__device__ __forceinline__ void dif32_stage(const float2* x, C2* ab) {
+  if constexpr (K < 16) {
+    const float2 a = cadd(x[K], x[K + 16]), d = csub(x[K], x[K + 16]);
+    constexpr float c = (float)cos32(K), s = (float)sin32(K);
+    float2 b;
+    if constexpr (K == 0) b = d;
+    else if constexpr (K == 8) b = make_float2(d.y, -d.x);
+    else b = make_float2(fmaf(c, d.x, s * d.y), fmaf(c, d.y, -s * d.x));
+    ab[K] = {make_float2(a.x, b.x), make_float2(a.y, b.y)};
+    dif32_stage<K + 1>(x, ab);
+  }
+}
+__device__ __forceinline__ void fft32_dif(const float2 (&x)[32], C2 (&X)[16]) {
+  C2 ab[16];
+  dif32_stage<0>(x, ab);
+  fft<16, 1, false>(ab, X);
+}
+template <int K>
+__device__ __forceinline__ void dit32_stage(const C2* eo, float2* x) {
+  if constexpr (K < 16) {
+    butterfly<32, K, true>(make_float2(eo[K].re.x, eo[K].im.x), make_float2(eo[K].re.y, eo[K].im.y), x[K], x[K + 16]);
+    dit32_stage<K + 1>(eo, x);
+  }
+}
+__device__ __forceinline__ void ifft32_dit(const C2 (&X)[16], float2 (&x)[32]) {
+  C2 eo[16];
+  fft<16, 1, true>(X, eo);
+  dit32_stage<0>(eo, x);
 }
 
 }  // namespace msp

@@ -1,97 +1,38 @@
-// msp_position.cu -- the fused per-position multislice forward / adjoint kernel.
+// msp_position.cu -- the fused per-position multislice forward / adjoint kernels (W = 64, 128).
 //
 // One CTA owns one scan position at a time (persistent grid, positions
-// s = blockIdx.x, blockIdx.x + gridDim.x, ...).  The W x W complex wave stays
-// in shared memory for the whole position: every slice's transmit (Sec. 2.1,
-// E_m = V_z(E_{m-1}) o X_m), Fresnel propagation F^-1(H o F .) and the far-field
-// transform F(E_M) run on it in place, then the amplitude-flow residual
-// (Sec. 3.2) and the adjoint recursion chi_{m-1} = G^H (conj(X_m) o chi_m)
-// (Sec. 3.3, the prefix / suffix products R_l and S_l applied matrix-free).
-//
-// Each eight-thread line group owns a small padded exchange buffer next to the
-// wave, so the in-line exchange never touches the wave itself.
-//
-// A propagation is  rows F -> [columns F, x H, columns F^-1] -> rows F^-1: the
-// column transforms and the propagator run back to back in registers, and the
-// inverse row transform of one slice, the transmit of the next slice and its
-// forward row transform also run back to back in registers.  Each phase is one
-// read and one write of the wave in shared memory plus the in-line exchange.
+// s = blockIdx.x, blockIdx.x + gridDim.x, ...) and runs the whole of it: every slice's
+// transmit (Sec. 2.1, E_m = V_z(E_{m-1}) o X_m), Fresnel propagation F^-1(H o F .), the
+// far-field transform F(E_M), the amplitude-flow residual (Sec. 3.2) and the adjoint
+// recursion chi_{m-1} = G^H (conj(X_m) o chi_m) (Sec. 3.3, the prefix / suffix products R_l
+// and S_l applied matrix-free).
 //
 // The propagator is separable, h(ky, kx) = h1(ky) h1(kx) with
 // h1(k) = exp(-i pi dz lambda q_k^2) / W (the 1/W^2 of F^-1 folded in), so it is
-// a W-entry shared table.  Global operands of a phase (transmission window,
-// measured intensities, stashed exit waves) are loaded before the line transform
-// that precedes their use, so their latency hides behind the arithmetic.
+// a W-entry shared table.
 //
 // The only per-slice global traffic is the transmission window (read), the exit
 // wave of each slice (written to this CTA's stash slot on the way forward, read
 // back on the way down; the slots are reused position after position so they
 // stay L2-resident) and the per-position window gradient.  The data each position
-// touches once (measured pattern, window gradients, illumination) is loaded and
-// stored with the evict-first (streaming) cache hint, so that it does not push the
-// stash slots out of L2.
+// touches once (window gradients, illumination) is stored with the evict-first
+// (streaming) cache hint, so that it does not push the stash slots out of L2.
+#include <type_traits>
+
 #include "msp_fft.cuh"
 #include "msp_kernels.cuh"
 #include "msp_tc.cuh"
 
-// Twiddles of the line transforms from shared memory (0) or registers (1).
-#ifndef MSP_TWIDDLE_REGISTERS
-#define MSP_TWIDDLE_REGISTERS 1
-#endif
-// In-line exchange with row-major (0) or transposed (1) step-A results.
-#ifndef MSP_TRANSPOSED_EXCHANGE
-#define MSP_TRANSPOSED_EXCHANGE 1
-#endif
-
 namespace msp {
 
-// Exit-wave stash in tensor memory (W = 128, one CTA per SM).  The fused kernel issues no MMAs,
-// so the SM's 256 KB of tensor memory is free: each thread keeps the values it stashes for two
-// slices in its own TMEM lane (warp w: lanes 32 (w % 4) .., columns 128 (w / 4) .. + 127; a
-// slice takes 2 row iterations x 16 complex values = 64 columns).  Those slices neither pass
-// through the L1 data pipe nor compete for L2 with the streaming window gradients; the others
-// use the CTA's global stash slot.  Loss and gradients: the last two slices (the first ones
-// the adjoint reads back); layer step: the one stashed slice.
-#ifndef MSP_TMEM_STASH
-#define MSP_TMEM_STASH 1
-#endif
-struct TmemStash {
-  uint32_t base;   // this thread's lane and its warp's first column
-  // 16 complex values of row iteration `it` of stash slot `slot` (0 or 1)
-  __device__ __forceinline__ uint32_t addr(int slot, int it) const { return base + (uint32_t)(64 * slot + 32 * it); }
-  __device__ __forceinline__ void store(int slot, int it, const float2 (&v)[16]) const {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(addr(slot, it)),
-        "f"(v[0].x), "f"(v[0].y), "f"(v[1].x), "f"(v[1].y), "f"(v[2].x), "f"(v[2].y), "f"(v[3].x), "f"(v[3].y),
-        "f"(v[4].x), "f"(v[4].y), "f"(v[5].x), "f"(v[5].y), "f"(v[6].x), "f"(v[6].y), "f"(v[7].x), "f"(v[7].y),
-        "f"(v[8].x), "f"(v[8].y), "f"(v[9].x), "f"(v[9].y), "f"(v[10].x), "f"(v[10].y), "f"(v[11].x), "f"(v[11].y),
-        "f"(v[12].x), "f"(v[12].y), "f"(v[13].x), "f"(v[13].y), "f"(v[14].x), "f"(v[14].y), "f"(v[15].x),
-        "f"(v[15].y)
-        : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-  }
-  __device__ __forceinline__ void load(int slot, int it, float2 (&v)[16]) const {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x),
-          "=f"(v[3].y), "=f"(v[4].x), "=f"(v[4].y), "=f"(v[5].x), "=f"(v[5].y), "=f"(v[6].x), "=f"(v[6].y),
-          "=f"(v[7].x), "=f"(v[7].y), "=f"(v[8].x), "=f"(v[8].y), "=f"(v[9].x), "=f"(v[9].y), "=f"(v[10].x),
-          "=f"(v[10].y), "=f"(v[11].x), "=f"(v[11].y), "=f"(v[12].x), "=f"(v[12].y), "=f"(v[13].x), "=f"(v[13].y),
-          "=f"(v[14].x), "=f"(v[14].y), "=f"(v[15].x), "=f"(v[15].y)
-        : "r"(addr(slot, it))
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-  }
-};
-
-#if MSP_TRANSPOSED_EXCHANGE
-#define LINE_FFT line_fft_t
-#else
-#define LINE_FFT line_fft
-#endif
-
+// ----------------------------------------------------------------------------
+// W = 64: the wave in shared memory, line transforms by groups of eight threads
+// ----------------------------------------------------------------------------
+// A propagation is  rows F -> [columns F, x H, columns F^-1] -> rows F^-1: the column transforms and
+// the propagator run back to back in registers, and the inverse row transform of one slice, the
+// transmit of the next slice and its forward row transform also run back to back in registers.
+// Each phase is one read and one write of the wave in shared memory plus the in-line exchange, which
+// goes through a small padded buffer that each line group owns next to the wave.
 template <int W>
 struct Geo {
   static constexpr int NT = 4 * W;        // threads per CTA
@@ -124,7 +65,7 @@ struct ColIdx {
 // Dynamic shared memory: the wave, then one exchange buffer per eight-thread line group.
 template <int W>
 __host__ __device__ constexpr int exchange_floats2() {
-  return MSP_TRANSPOSED_EXCHANGE ? kXGroup(W / 8) : 8 * (W / 8 + 1);
+  return kXGroup(W / 8);
 }
 template <int W>
 constexpr size_t position_smem_bytes() {
@@ -158,35 +99,13 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
   }
   if (tid < W) s_h1[tid] = p.h1[tid];
   __syncthreads();
-#if MSP_TWIDDLE_REGISTERS
   const RegisterTwiddles<W, 8> tw(s_tw, j);
-#else
-  const SharedTwiddles<8> tw{s_tw, j};
-#endif
 
   const int L = p.L;
   const float zthr2 = (MODE == MODE_FORWARD) ? 0.f : (float)p.zthr2[0];
   const bool need_stash = (MODE == MODE_LOSS_GRAD && !p.loss_only) || (MODE == MODE_LAYER);
   const int lowest = (MODE == MODE_LAYER) ? p.layer : 0;
   bool first_dprobe = true;
-  // TMEM stash (W = 128 only): slot of slice l, or -1 for the global stash
-  constexpr bool kTmem = MSP_TMEM_STASH && W == 128 && (MODE == MODE_LOSS_GRAD || MODE == MODE_LAYER);
-  __shared__ uint32_t s_tmem;
-  TmemStash ts{0};
-  if constexpr (kTmem) {
-    if (tid < 32) tc::tmem_alloc(&s_tmem, 512);
-    tc::fence_before();
-    __syncthreads();
-    tc::fence_after();
-    const int warp = tid >> 5;
-    ts.base = s_tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(128 * (warp >> 2));
-  }
-  auto tslot = [&](int l) -> int {
-    if constexpr (!kTmem) return -1;
-    if (MODE == MODE_LAYER) return 0;
-    return l >= L - 2 ? l - (L - 2 > 0 ? L - 2 : 0) : -1;
-  };
-
   for (int s = blockIdx.x; s < p.S; s += gridDim.x) {
     const int2 ps = p.pos[s];
     const int y0 = ps.x, x0 = ps.y;
@@ -221,26 +140,16 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
       for (int m = 0; m < N1; ++m) v[m] = p.probe[r * W + j + 8 * m];
       const bool keep0 = need_stash && (MODE == MODE_LOSS_GRAD || p.layer == 0);
       if (CPLX && keep0) {
-        if constexpr (kTmem) {
-          if (tslot(0) >= 0) ts.store(tslot(0), it, v);   // incident wave
-        }
-        if (tslot(0) < 0) {
 #pragma unroll
-          for (int m = 0; m < N1; ++m) stash[r * W + j + 8 * m] = v[m];   // incident wave
-        }
+        for (int m = 0; m < N1; ++m) stash[r * W + j + 8 * m] = v[m];   // incident wave
       }
 #pragma unroll
       for (int m = 0; m < N1; ++m) v[m] = cmul(v[m], T0[j + 8 * m]);
       if (!CPLX && keep0) {
-        if constexpr (kTmem) {
-          if (tslot(0) >= 0) ts.store(tslot(0), it, v);   // exit wave
-        }
-        if (tslot(0) < 0) {
 #pragma unroll
-          for (int m = 0; m < N1; ++m) stash[r * W + j + 8 * m] = v[m];   // exit wave
-        }
+        for (int m = 0; m < N1; ++m) stash[r * W + j + 8 * m] = v[m];   // exit wave
       }
-      LINE_FFT<W, false>(v, tw, xb, j);
+      line_fft_t<W, false>(v, tw, xb, j);
 #pragma unroll
       for (int m = 0; m < N1; ++m) sm[RowIdx<W>(r, j)(m)] = v[m];
     }
@@ -258,11 +167,11 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
           float2 v[N1];
 #pragma unroll
           for (int m = 0; m < N1; ++m) v[m] = sm[ca(m)];
-          LINE_FFT<W, false>(v, tw, xb, j);
+          line_fft_t<W, false>(v, tw, xb, j);
           const float2 hx = s_h1[c];
 #pragma unroll
           for (int m = 0; m < N1; ++m) v[m] = cmul(v[m], cmul(s_h1[j + 8 * m], hx));
-          LINE_FFT<W, true>(v, tw, xb, j);
+          line_fft_t<W, true>(v, tw, xb, j);
 #pragma unroll
           for (int m = 0; m < N1; ++m) sm[ca(m)] = v[m];
         }
@@ -281,28 +190,18 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
           for (int m = 0; m < N1; ++m) t[m] = Tr[j + 8 * m];     // in flight during the transform
 #pragma unroll
           for (int m = 0; m < N1; ++m) v[m] = sm[ra(m)];
-          LINE_FFT<W, true>(v, tw, xb, j);
+          line_fft_t<W, true>(v, tw, xb, j);
           if (CPLX && keep) {
-            if constexpr (kTmem) {
-              if (tslot(l + 1) >= 0) ts.store(tslot(l + 1), it, v);   // incident wave
-            }
-            if (tslot(l + 1) < 0) {
 #pragma unroll
-              for (int m = 0; m < N1; ++m) st[r * W + j + 8 * m] = v[m];   // incident wave
-            }
+            for (int m = 0; m < N1; ++m) st[r * W + j + 8 * m] = v[m];   // incident wave
           }
 #pragma unroll
           for (int m = 0; m < N1; ++m) v[m] = cmul(v[m], t[m]);
           if (!CPLX && keep) {
-            if constexpr (kTmem) {
-              if (tslot(l + 1) >= 0) ts.store(tslot(l + 1), it, v);   // exit wave
-            }
-            if (tslot(l + 1) < 0) {
 #pragma unroll
-              for (int m = 0; m < N1; ++m) st[r * W + j + 8 * m] = v[m];   // exit wave
-            }
+            for (int m = 0; m < N1; ++m) st[r * W + j + 8 * m] = v[m];   // exit wave
           }
-          LINE_FFT<W, false>(v, tw, xb, j);
+          line_fft_t<W, false>(v, tw, xb, j);
 #pragma unroll
           for (int m = 0; m < N1; ++m) sm[ra(m)] = v[m];
         }
@@ -322,27 +221,17 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
           }
 #pragma unroll
           for (int m = 0; m < N1; ++m) v[m] = sm[ca(m)];
-          LINE_FFT<W, false>(v, tw, xb, j);
+          line_fft_t<W, false>(v, tw, xb, j);
           if (MODE == MODE_FORWARD) {
             float* out = p.I_out + s * WW + c;
 #pragma unroll
             for (int m = 0; m < N1; ++m) out[(j + 8 * m) * W] = fmaf(v[m].x, v[m].x, v[m].y * v[m].y);
           } else {
             // amplitude-flow residual R = Psi - sqrt(I) Psi / |Psi| (fraction 0 where Psi counts as 0)
-#pragma unroll
-            for (int m = 0; m < N1; ++m) {
-              const float a2 = fmaf(v[m].x, v[m].x, v[m].y * v[m].y);
-              const float a = sqrtf(a2);
-              const float rt = sqrtf(im[m]);
-              const float d = rt - a;
-              lsum = fmaf(d, d, lsum);
-              // below the threshold the fraction is 0, so R = Psi (f = 1); a2 > zthr2 >= 0 implies a > 0
-              const float f = (a2 > zthr2) ? (1.f - rt / a) : 1.f;
-              v[m] = make_float2(v[m].x * f, v[m].y * f);
-            }
+            residual(v, im, zthr2, lsum);
             // chi = F^H R: inverse column transforms now, rows below
             if (!p.loss_only) {
-              LINE_FFT<W, true>(v, tw, xb, j);
+              line_fft_t<W, true>(v, tw, xb, j);
 #pragma unroll
               for (int m = 0; m < N1; ++m) sm[ca(m)] = v[m];
             }
@@ -382,17 +271,12 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
         const RowIdx<W> ra(r, j);
         float2 e[N1], v[N1];
         if (grad_here) {
-          if constexpr (kTmem) {
-            if (tslot(l) >= 0) ts.load(tslot(l), it, e);
-          }
-          if (tslot(l) < 0) {
 #pragma unroll
-            for (int m = 0; m < N1; ++m) e[m] = st[r * W + j + 8 * m];   // in flight during the transform
-          }
+          for (int m = 0; m < N1; ++m) e[m] = st[r * W + j + 8 * m];   // in flight during the transform
         }
 #pragma unroll
         for (int m = 0; m < N1; ++m) v[m] = sm[ra(m)];
-        LINE_FFT<W, true>(v, tw, xb, j);   // v = chi_l (row r)
+        line_fft_t<W, true>(v, tw, xb, j);   // v = chi_l (row r)
         if (grad_here) {
           // object-frame offset of this row's first element (the layer step's map is one slice)
           const size_t o = (MODE == MODE_LOSS_GRAD ? (size_t)l * plane : 0) + win0 + (size_t)r * p.Nx + j;
@@ -439,7 +323,7 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
               for (int m = 0; m < N1; ++m) dp[j + 8 * m] = cadd(dp[j + 8 * m], v[m]);
             }
           } else {
-            LINE_FFT<W, false>(v, tw, xb, j);
+            line_fft_t<W, false>(v, tw, xb, j);
 #pragma unroll
             for (int m = 0; m < N1; ++m) sm[ra(m)] = v[m];
           }
@@ -456,11 +340,11 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
         float2 v[N1];
 #pragma unroll
         for (int m = 0; m < N1; ++m) v[m] = sm[ca(m)];
-        LINE_FFT<W, false>(v, tw, xb, j);
+        line_fft_t<W, false>(v, tw, xb, j);
         const float2 hx = s_h1[c];
 #pragma unroll
         for (int m = 0; m < N1; ++m) v[m] = cmulc(v[m], cmul(s_h1[j + 8 * m], hx));
-        LINE_FFT<W, true>(v, tw, xb, j);
+        line_fft_t<W, true>(v, tw, xb, j);
 #pragma unroll
         for (int m = 0; m < N1; ++m) sm[ca(m)] = v[m];
       }
@@ -474,7 +358,606 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
     float2* dp = p.dprobe_part + (size_t)blockIdx.x * WW;
     for (size_t i = tid; i < WW; i += G::NT) dp[i] = make_float2(0.f, 0.f);
   }
-  if constexpr (kTmem) {
+}
+
+// ----------------------------------------------------------------------------
+// W = 128: the wave in registers, two values per packed instruction
+// ----------------------------------------------------------------------------
+// 512 threads hold the wave, 32 complex values each; shared memory only carries it from one pass to the
+// next.  The 2-D transform is split over the two axes together, with row n = 16 n1 + n2 and column
+// n = 32 n1 + n2 (four-step Cooley-Tukey per axis; spectrum index k1 + 8 k2 and k1 + 4 k2):
+//   pass A   the 8-point row and 4-point column transforms over the two n1.  The warp is the row's n2, the
+//            lane the column's n2: every global access (transmission window, window gradients) is a run
+//            of 32 consecutive elements of a row;
+//   pass B   the 32-point column transform over the column's n2, one row of 32 values per thread;
+//   pass C   the 16-point row transform over the row's n2 of two columns per thread, the propagator (or the
+//            far field and its residual), and the inverse 16-point transform.
+// The inverse runs B, A.  A row's n2 stays with its warp from B through A to B, so these exchanges need warp
+// synchronisation only, within the warp's own region; the CTA meets at the two sides of pass C.  Every pass
+// writes back to the addresses that it read.  Spectra stay in the order of the split: the propagator and
+// the patterns are indexed by k, and the inverse consumes the same order.
+//
+// Against line transforms of eight threads with an exchange inside each (the form below W = 64 still uses),
+// a propagation moves the wave through shared memory four times in and out instead of six, and packed
+// arithmetic needs 313 thousand warp instructions per position (W = 128, L = 4) instead of 441.  What bounds
+// it: the L1 data pipe (61 %), the FP32 pipe (48 %) and issue (46 %) together, with the warps of a
+// position in step between two barriers.  Loss and gradients, W = 128, L = 4, 1024 positions: 0.709 -> 0.587
+// ms; forward model 0.302 -> 0.251 ms; L = 8, 4096 positions: 5.68 -> 4.77 ms.
+namespace w128 {
+constexpr int W = 128, NT = 512;
+constexpr int RH = 8, RL = 16, CH = 4, CL = 32, V = 32;
+constexpr int XS = CL + 2;          // row stride of a region (float2)
+constexpr int REGION = V * XS;
+constexpr int TBUF = 16;            // transmission values per thread that are fetched a pass ahead
+constexpr size_t SMEM = ((size_t)RL * REGION + (size_t)TBUF * NT) * sizeof(float2);
+
+__device__ __forceinline__ void fetch8(float2* dst, const float2* src) {   // 8 bytes, asynchronously
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void fetch4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void fetch_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Half a slice of a thread's values (16 complex) in its own TMEM lane.
+__device__ __forceinline__ void tmem_store(uint32_t addr, const C2 (&v)[8]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(addr),
+      "f"(v[0].re.x), "f"(v[0].re.y), "f"(v[0].im.x), "f"(v[0].im.y), "f"(v[1].re.x), "f"(v[1].re.y), "f"(v[1].im.x),
+      "f"(v[1].im.y), "f"(v[2].re.x), "f"(v[2].re.y), "f"(v[2].im.x), "f"(v[2].im.y), "f"(v[3].re.x), "f"(v[3].re.y),
+      "f"(v[3].im.x), "f"(v[3].im.y), "f"(v[4].re.x), "f"(v[4].re.y), "f"(v[4].im.x), "f"(v[4].im.y), "f"(v[5].re.x),
+      "f"(v[5].re.y), "f"(v[5].im.x), "f"(v[5].im.y), "f"(v[6].re.x), "f"(v[6].re.y), "f"(v[6].im.x), "f"(v[6].im.y),
+      "f"(v[7].re.x), "f"(v[7].re.y), "f"(v[7].im.x), "f"(v[7].im.y)
+      : "memory");
+}
+__device__ __forceinline__ C2 tmem_c2(const uint32_t* r) {
+  return {make_float2(__uint_as_float(r[0]), __uint_as_float(r[1])), make_float2(__uint_as_float(r[2]), __uint_as_float(r[3]))};
+}
+// four values of each column of the half slice at `addr`
+__device__ __forceinline__ void tmem_load(uint32_t addr, C2 (&v)[4]) {
+  uint32_t r[16];
+  tc::tmem_ld16(addr, r);
+  tc::tmem_wait_ld();
+  tc::tmem_ready(r);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = tmem_c2(r + 4 * i);
+}
+// A value that the compiler has to take as new here: what is derived from it is derived again instead of
+// being kept in registers across the passes.
+__device__ __forceinline__ uint32_t anew(uint32_t a) {
+  asm volatile("" : "+r"(a));
+  return a;
+}
+// a & b, tested anew at each use
+__device__ __forceinline__ bool word(uint32_t a, uint32_t b) {
+  return (anew(a) & b) != 0;
+}
+}  // namespace w128
+
+template <int MODE, bool CPLX>
+__global__ void __launch_bounds__(512, 1) position_kernel_128(const PosParams p) {
+  using namespace w128;
+  extern __shared__ float4 sm4[];
+  float2* sm = reinterpret_cast<float2*>(sm4);
+  __shared__ float2 s_w[W];     // w_W^k
+  __shared__ float4 s_wd[W];    // the same, (re, re, im, im)
+  __shared__ float2 s_h1[W];    // h1(k) = exp(-i pi dz lambda q_k^2) / W
+  __shared__ float4 s_hd[W];    // the same, (re, re, im, im)
+  __shared__ float red[NT / 32];
+  __shared__ float s_zthr2;
+  __shared__ int2 s_pos[2];     // window origins of this CTA's positions, the j-th one in s_pos[j & 1]
+  __shared__ uint32_t s_tmem;
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = (int)anew(tid >> 5);
+  constexpr size_t WW = (size_t)W * W;
+  const size_t plane = (size_t)p.Ny * p.Nx;
+
+  if (tid < W) {   // evaluated in double, rounded once
+    double sn, cs;
+    sincospi(2.0 * (double)tid / (double)W, &sn, &cs);
+    const float2 w = make_float2((float)cs, (float)-sn), h = p.h1[tid];
+    s_w[tid] = w;
+    s_wd[tid] = make_float4(w.x, w.x, w.y, w.y);
+    s_h1[tid] = h;
+    s_hd[tid] = make_float4(h.x, h.x, h.y, h.y);
+  }
+  if (MODE != MODE_FORWARD && tid == 0) s_zthr2 = (float)p.zthr2[0];
+  if (tid < 2) {
+    const int sp = blockIdx.x + tid * gridDim.x;
+    s_pos[tid] = sp < p.S ? p.pos[sp] : make_int2(-1, -1);
+  }
+  constexpr bool kStash = MODE == MODE_LOSS_GRAD || MODE == MODE_LAYER;
+  uint32_t tm = 0;   // this thread's TMEM lane and its warp's first column
+  if constexpr (kStash) {
+    if (tid < 32) tc::tmem_alloc(&s_tmem, 512);
+    tc::fence_before();
+  }
+  __syncthreads();
+  if constexpr (kStash) {
+    tc::fence_after();
+    tm = s_tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(128 * (warp >> 2));
+  }
+
+  // passes A and B: the row's n2 is the warp, in A the column's n2 the lane
+  float2* const sa = sm + warp * REGION + lane;           // A: value a at sa[a XS]
+  float2* const sb = sm + warp * REGION + lane * XS;      // B: this thread's row
+  float2* const tb = sm + RL * REGION + tid;              // fetched transmissions: value i at tb[i NT]
+  const int rc = warp * W + lane;                         // window offset of value (0, 0) in pass A
+  // pass C: spectrum row k1r + RH k2, columns kc and kc + CH
+  const int k1r = warp & 7, k1c = lane >> 3, xp = (lane & 7) + 8 * (warp >> 3);
+  float2* const sc = sm + (CH * k1r + k1c) * XS + 2 * xp; // C: row n2 at sc[n2 REGION]
+  const int kc = k1c + CH * 2 * xp;
+
+  const int L = p.L;
+  const bool need_stash = (MODE == MODE_LOSS_GRAD && !p.loss_only) || (MODE == MODE_LAYER);
+  const int lowest = (MODE == MODE_LAYER) ? p.layer : 0;
+  // TMEM slot (32 columns) of half h of slice l, or -1 for the global stash: there is room for four halves
+  auto half_slot = [&](int l, int h) -> int {
+    if (MODE == MODE_LAYER) return h;
+    if (L <= 2) return 2 * l + h;
+    return (h == 0 && l >= L - 4) ? l - (L > 4 ? L - 4 : 0) : -1;
+  };
+  // keeps the exit (or incident) wave of half h of slice l for the adjoint; the thread that wrote it reads it
+  // back, so the pairs are kept as they are, 16 bytes per lane
+  auto keep_half = [&](int l, int h, float4* st, const C2 (&q)[8]) {
+    const int sl = half_slot(l, h);
+    if (sl >= 0) {
+      tmem_store(tm + 32u * sl, q);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) st[(8 * h + i) * NT + tid] = make_float4(q[i].re.x, q[i].re.y, q[i].im.x, q[i].im.y);
+    }
+  };
+
+  // forward pass A behind the row transforms: v[half][k1r] -> shared memory
+  auto a_out = [&](const C2 (&v)[2][8]) {
+    const uint32_t cl = anew(lane);
+    const float2 w1 = s_w[cl], w2 = s_w[2 * cl], w3 = s_w[3 * cl];   // column twiddles w_W^(n2 k1)
+#pragma unroll
+    for (int h = 0; h < RH; ++h) {
+      C2 a = v[0][h], b = v[1][h];
+      if (h) {   // row twiddle w_W^(n2 k1)
+        const float4 w = s_wd[warp * h];
+        const float2 wx = make_float2(w.x, w.y), wy = make_float2(w.z, w.w);
+        a = {sub2(mul2(a.re, wx), mul2(a.im, wy)), fma2(a.re, wy, mul2(a.im, wx))};
+        b = {sub2(mul2(b.re, wx), mul2(b.im, wy)), fma2(b.re, wy, mul2(b.im, wx))};
+      }
+      // four-point column transform: (E, O) sums and differences in pairs, then scalars
+      const C2 s = add(a, b), d = sub(a, b);
+      const float2 y0 = make_float2(s.re.x + s.re.y, s.im.x + s.im.y);
+      const float2 y2 = make_float2(s.re.x - s.re.y, s.im.x - s.im.y);
+      const float2 y1 = make_float2(d.re.x + d.im.y, d.im.x - d.re.y);
+      const float2 y3 = make_float2(d.re.x - d.im.y, d.im.x + d.re.y);
+      sa[(h * CH + 0) * XS] = y0;
+      sa[(h * CH + 1) * XS] = cmul(y1, w1);
+      sa[(h * CH + 2) * XS] = cmul(y2, w2);
+      sa[(h * CH + 3) * XS] = cmul(y3, w3);
+    }
+  };
+  // inverse pass A up to the row transforms: shared memory -> v[half][k1r]
+  auto a_in = [&](C2 (&v)[2][8]) {
+    const uint32_t cl = anew(lane);
+    const float2 w1 = s_w[cl], w2 = s_w[2 * cl], w3 = s_w[3 * cl];
+#pragma unroll
+    for (int h = 0; h < RH; ++h) {
+      const float2 t0 = sa[(h * CH + 0) * XS];
+      const float2 t1 = cmulc(sa[(h * CH + 1) * XS], w1);
+      const float2 t2 = cmulc(sa[(h * CH + 2) * XS], w2);
+      const float2 t3 = cmulc(sa[(h * CH + 3) * XS], w3);
+      // (E0, E1) and (O0, i O1)
+      const C2 e = {make_float2(t0.x + t2.x, t0.x - t2.x), make_float2(t0.y + t2.y, t0.y - t2.y)};
+      const C2 o = {make_float2(t1.x + t3.x, t3.y - t1.y), make_float2(t1.y + t3.y, t1.x - t3.x)};
+      C2 a = add(e, o), b = sub(e, o);
+      if (h) {
+        const float4 w = s_wd[warp * h];
+        const float2 wx = make_float2(w.x, w.y), wy = make_float2(w.z, w.w);
+        a = {fma2(a.re, wx, mul2(a.im, wy)), sub2(mul2(a.im, wx), mul2(a.re, wy))};
+        b = {fma2(b.re, wx, mul2(b.im, wy)), sub2(mul2(b.im, wx), mul2(b.re, wy))};
+      }
+      v[0][h] = a;
+      v[1][h] = b;
+    }
+  };
+
+  // q o X of half u of a window (q o conj(X) on the way back)
+  auto transmit = [&](auto conj, int u, C2 (&q)[8]) {
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      const float2 x0 = u == 0 ? tb[(2 * h) * NT] : sa[(2 * h) * XS], x1 = u == 0 ? tb[(2 * h + 1) * NT] : sa[(2 * h + 1) * XS];
+      const float2 q0 = make_float2(q[h].re.x, q[h].im.x), q1 = make_float2(q[h].re.y, q[h].im.y);
+      const float2 y0 = conj.value ? cmulc(q0, x0) : cmul(q0, x0), y1 = conj.value ? cmulc(q1, x1) : cmul(q1, x1);
+      q[h] = {make_float2(y0.x, y1.x), make_float2(y0.y, y1.y)};
+    }
+  };
+  constexpr std::false_type kPlain{};
+  constexpr std::true_type kConj{};
+
+  constexpr uint32_t kForward = 1, kKeep = 2, kGrad = 4, kGoOn = 8, kPropagate = 16;   // words of a pass
+  // The object offset of a window's origin (a plane holds at most 4e9 values), or kNoWindow.
+  constexpr uint32_t kNoWindow = 0xffffffffu;
+  auto window = [&](uint32_t j) {
+    const int2 ps = s_pos[j & 1];
+    const bool ok = ps.x >= 0 && ps.y >= 0 && ps.x <= p.Ny - W && ps.y <= p.Nx - W;
+    return ok ? (uint32_t)ps.x * (uint32_t)p.Nx + (uint32_t)ps.y : kNoWindow;
+  };
+  // Transmission windows arrive asynchronously: the first half of a slice's (column groups 0 and 1) in tb,
+  // fetched a pass ahead; the second half in this thread's slots of the wave, which are free between
+  // a_in and a_out.  Each thread fetches what it uses itself, so no other synchronisation is needed.
+  auto fetch_first = [&](const float2* T) {
+    const size_t hstep = (size_t)RL * anew(p.Nx);
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      fetch8(tb + (2 * h) * NT, T + h * hstep);
+      fetch8(tb + (2 * h + 1) * NT, T + h * hstep + CL);
+    }
+  };
+  auto fetch_second = [&](const float2* T) {
+    const size_t hstep = (size_t)RL * anew(p.Nx);
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      fetch8(sa + (2 * h) * XS, T + h * hstep + 2 * CL);
+      fetch8(sa + (2 * h + 1) * XS, T + h * hstep + 3 * CL);
+    }
+  };
+
+  // the window gradient of values 4 i .. 4 i + 3 of half u of slice l from chi_l = q and the stashed wave e
+  auto gradient = [&](int s, int l, int u, int i, uint32_t oc, const C2* q, const C2 (&e)[4]) {
+    // window gradients: [S][L][W][W] (LOSS_GRAD) or [S][W][W] (LAYER), float2 in transmission mode
+    const size_t wo = (MODE == MODE_LOSS_GRAD ? ((size_t)s * L + l) * WW : (size_t)s * WW) + rc + RL * 4 * i * W + CL * 2 * u;
+    // object-frame offset (the layer step's map is one slice)
+    const size_t hstep = (size_t)RL * anew(p.Nx);
+    const size_t om = (MODE == MODE_LOSS_GRAD ? (size_t)l * plane : 0) + oc + 4 * i * hstep + CL * 2 * u;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      if (CPLX) {   // dL/dconj(o_l) on the window: conj(psi_in,l) o chi_l
+        const float2 a = cmulc(make_float2(q[h].re.x, q[h].im.x), make_float2(e[h].re.x, e[h].im.x));
+        const float2 b = cmulc(make_float2(q[h].re.y, q[h].im.y), make_float2(e[h].re.y, e[h].im.y));
+        if (p.dVred) {   // reductions in L2
+          atomicAdd(reinterpret_cast<float2*>(p.dVred) + om + h * hstep, a);
+          atomicAdd(reinterpret_cast<float2*>(p.dVred) + om + h * hstep + CL, b);
+        } else {
+          __stcs(reinterpret_cast<float2*>(p.wgrad) + wo + RL * h * W, a);
+          __stcs(reinterpret_cast<float2*>(p.wgrad) + wo + RL * h * W + CL, b);
+        }
+      } else {      // dL/dV_l on the window: 2 sigma Im(conj(E_l) chi_l)
+        const float2 d = mul2(make_float2(p.two_sigma, p.two_sigma), sub2(mul2(e[h].re, q[h].im), mul2(e[h].im, q[h].re)));
+        if (p.dVred) {
+          atomicAdd(p.dVred + om + h * hstep, d.x);
+          atomicAdd(p.dVred + om + h * hstep + CL, d.y);
+        } else {
+          __stcs(p.wgrad + wo + RL * h * W, d.x);
+          __stcs(p.wgrad + wo + RL * h * W + CL, d.y);
+        }
+      }
+      if (MODE == MODE_LAYER) {   // |psi_in,l|^2 (= |E_l|^2 for unimodular slices)
+        const float2 d = fma2(e[h].re, e[h].re, mul2(e[h].im, e[h].im));
+        if (p.illumred) {
+          atomicAdd(p.illumred + om + h * hstep, d.x);
+          atomicAdd(p.illumred + om + h * hstep + CL, d.y);
+        } else {
+          __stcs(p.willum + wo + RL * h * W, d.x);
+          __stcs(p.willum + wo + RL * h * W + CL, d.y);
+        }
+      }
+    }
+  };
+
+  // State carried from position to position: the lowest bit, the parity of the position's number in this CTA;
+  // kFetched, slice 0 of the coming position is under way; kSummed, this CTA's probe-gradient partial has been
+  // written.  Like the words of a pass it is tested where it is used: flags that live across a pass cost
+  // registers, and the few that do not fit go to local memory at L2 latency (measured: 722 bytes of spills
+  // made the loss-and-gradient pass 1.16 times as long as 230 bytes).
+  constexpr uint32_t kFetched = 2, kSummed = 4;
+  uint32_t state = 0;
+  auto fetch_next_first = [&]() {
+    const uint32_t at = window(state + 1);
+    if (at != kNoWindow) fetch_first(p.T + (at + (uint32_t)warp * (uint32_t)p.Nx + (uint32_t)lane));
+  };
+  auto fetch_next_second = [&]() {
+    const uint32_t at = window(state + 1);
+    if (at != kNoWindow) fetch_second(p.T + (at + (uint32_t)warp * (uint32_t)p.Nx + (uint32_t)lane));
+  };
+  // the origin after the next one into this position's slot; tid 0 waits for it in its next slice 0, and the
+  // barriers that follow there show it to the others
+  auto fetch_origin = [&](int s) {
+    const int sp = s + 2 * (int)gridDim.x;
+    if (tid == 0 && sp < p.S) fetch8(reinterpret_cast<float2*>(&s_pos[state & 1]), reinterpret_cast<const float2*>(p.pos + sp));
+    if (tid == 0 && sp >= p.S) s_pos[state & 1] = make_int2(-1, -1);
+  };
+  for (int s = blockIdx.x; s < p.S; s += gridDim.x, state ^= 1) {
+    const uint32_t at = window(state);
+    if (at == kNoWindow) {
+      if (tid == 0) atomicMax(p.err, 1);
+      // outputs of a skipped position are zero
+      if (MODE == MODE_FORWARD) {
+        for (size_t i = tid; i < WW; i += NT) p.I_out[s * WW + i] = 0.f;
+      } else {
+        if (tid == 0) p.loss_part[s] = 0.0;
+        constexpr int CW = CPLX ? 2 : 1;
+        if (MODE == MODE_LOSS_GRAD && !p.dVred)
+          for (size_t i = tid; i < CW * WW * L; i += NT) p.wgrad[CW * s * WW * L + i] = 0.f;
+        if (MODE == MODE_LAYER && !p.dVred) {
+          for (size_t i = tid; i < CW * WW; i += NT) p.wgrad[CW * s * WW + i] = 0.f;
+          for (size_t i = tid; i < WW; i += NT) p.willum[s * WW + i] = 0.f;
+        }
+      }
+      state &= ~kFetched;
+      __syncthreads();   // every thread has read this position's slot
+      fetch_origin(s);
+      fetch_commit();
+      fetch_wait<0>();
+      __syncthreads();
+      continue;  // uniform across the CTA
+    }
+    const uint32_t oc = at + (uint32_t)warp * (uint32_t)p.Nx + (uint32_t)lane;   // object offset of this thread's value (0, 0)
+    float4* stash = reinterpret_cast<float4*>(p.stash + (size_t)blockIdx.x * (MODE == MODE_LOSS_GRAD ? L : 1) * WW);
+    const bool forward_only = MODE == MODE_FORWARD || p.loss_only;
+    // what the buffer tb receives after slice l's pass on the way forward: the next slice's window, or this
+    // thread's values of the measured pattern, or slice 0 of the next position
+    auto fetch_after = [&](int l) {
+      if (l + 1 < L) {
+        fetch_first(p.T + (size_t)(l + 1) * plane + oc);
+      } else if (MODE != MODE_FORWARD) {
+        const float* I = p.I_meas + s * WW + k1r * W + kc;
+#pragma unroll
+        for (int k = 0; k < RL; ++k) {
+          fetch4(&tb[k * NT].x, I + k * (RH * W));
+          fetch4(&tb[k * NT].y, I + k * (RH * W) + CH);
+        }
+      } else if (L > 1) {   // with one slice the next origin is not known yet
+        fetch_next_first();
+      }
+      fetch_commit();
+    };
+
+    C2 v[2][8];
+    {   // slice 0: probe o X_0, forward pass A
+      const bool keep = need_stash && (MODE == MODE_LOSS_GRAD || p.layer == 0);
+      if (!word(state, kFetched)) {
+        fetch_first(p.T + oc);
+        fetch_second(p.T + oc);
+        fetch_commit();
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        C2 q[8];
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+          const float2 a = p.probe[rc + RL * h * W + CL * 2 * u], b = p.probe[rc + RL * h * W + CL * (2 * u + 1)];
+          q[h] = {make_float2(a.x, b.x), make_float2(a.y, b.y)};
+        }
+        if (CPLX && keep) keep_half(0, u, stash, q);   // incident wave
+        if (u == 0) fetch_wait<0>();
+        transmit(kPlain, u, q);
+        if (u == 0) fetch_after(0);
+        if (!CPLX && keep) keep_half(0, u, stash, q);  // exit wave
+        fft<8, 1, false>(q, v[u]);
+      }
+      if constexpr (kStash) tc::tmem_wait_st();
+      a_out(v);
+    }
+
+    // step st < L - 1: propagate slice st to st + 1 and transmit; st = L - 1: far field, residual and the
+    // adjoint of slice L - 1; st >= L: back-propagate to slice l = 2 L - 2 - st and its adjoint
+#pragma unroll 1
+    for (int st = 0;; ++st) {
+      __syncwarp();
+      {   // ---------------- pass B ----------------
+        float4* q = reinterpret_cast<float4*>(sb);
+        float2 x[32];
+        C2 X[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float4 f = q[i];
+          x[2 * i] = make_float2(f.x, f.y);
+          x[2 * i + 1] = make_float2(f.z, f.w);
+        }
+        fft32_dif(x, X);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) q[i] = make_float4(X[i].re.x, X[i].re.y, X[i].im.x, X[i].im.y);
+      }
+      // ---------------- pass C ----------------
+      {
+        if (MODE != MODE_FORWARD && st == L - 1) fetch_wait<0>();   // the pattern
+        __syncthreads();
+        C2 x[16], X[16];
+#pragma unroll
+        for (int n = 0; n < RL; ++n) {
+          const float4 f = *reinterpret_cast<const float4*>(sc + n * REGION);
+          x[n] = {make_float2(f.x, f.y), make_float2(f.z, f.w)};
+        }
+        fft<16, 1, false>(x, X);
+        if (st != L - 1) {   // x H / W^2 (conjugated on the way back)
+          const float sg = st < L ? 1.f : -1.f;
+          const uint32_t c = anew(kc);
+          const float2 h0 = s_h1[c], h1 = s_h1[c + CH];
+          const float2 hcr = make_float2(h0.x, h1.x), hcn = make_float2(-h0.y, -h1.y);
+          const float2 hcrs = make_float2(sg * h0.x, sg * h1.x), hcis = make_float2(sg * h0.y, sg * h1.y);
+#pragma unroll
+          for (int k = 0; k < RL; ++k) {
+            const float4 h = s_hd[k1r + RH * k];
+            const float2 hx = make_float2(h.x, h.y), hy = make_float2(h.z, h.w);
+            const float2 pr = fma2(hx, hcr, mul2(hy, hcn)), pi = fma2(hx, hcis, mul2(hy, hcrs));
+            X[k] = {sub2(mul2(X[k].re, pr), mul2(X[k].im, pi)), fma2(X[k].re, pi, mul2(X[k].im, pr))};
+          }
+        } else if (MODE == MODE_FORWARD) {   // far field Psi
+#pragma unroll
+          for (int k = 0; k < RL; ++k) {
+            const float2 a2 = fma2(X[k].re, X[k].re, mul2(X[k].im, X[k].im));
+            float* out = p.I_out + s * WW + (k1r + RH * k) * W + kc;
+            out[0] = a2.x;
+            out[CH] = a2.y;
+          }
+        } else {   // far field, residual R = Psi - sqrt(I) Psi / |Psi|
+          const float zthr2 = s_zthr2;
+          float lsum = 0.f;
+          bool finite = true;
+#pragma unroll
+          for (int k = 0; k < RL; ++k) {
+            const float2 a2 = fma2(X[k].re, X[k].re, mul2(X[k].im, X[k].im));
+            finite = finite && residual_is_finite(a2.x, tb[k * NT].x) && residual_is_finite(a2.y, tb[k * NT].y);
+          }
+          if (finite) {
+#pragma unroll
+            for (int k = 0; k < RL; ++k) {
+              const float2 a2 = fma2(X[k].re, X[k].re, mul2(X[k].im, X[k].im));
+              const float2 im = tb[k * NT];
+              const float2 f = make_float2(residual_finite(a2.x, im.x, zthr2, lsum), residual_finite(a2.y, im.y, zthr2, lsum));
+              X[k] = {mul2(X[k].re, f), mul2(X[k].im, f)};
+            }
+          } else {   // through this thread's slots of the wave, to keep the rare path short
+#pragma unroll
+            for (int k = 0; k < RL; ++k)
+              *reinterpret_cast<float4*>(sc + k * REGION) = make_float4(X[k].re.x, X[k].re.y, X[k].im.x, X[k].im.y);
+#pragma unroll 1
+            for (int k = 0; k < RL; ++k) {
+              float4& f = *reinterpret_cast<float4*>(sc + k * REGION);
+              const float2 im = tb[k * NT];
+              const float fx = residual_exact(fmaf(f.x, f.x, f.z * f.z), im.x, zthr2, lsum);
+              const float fy = residual_exact(fmaf(f.y, f.y, f.w * f.w), im.y, zthr2, lsum);
+              f = make_float4(f.x * fx, f.y * fy, f.z * fx, f.w * fy);
+            }
+#pragma unroll
+            for (int k = 0; k < RL; ++k) {
+              const float4 f = *reinterpret_cast<const float4*>(sc + k * REGION);
+              X[k] = {make_float2(f.x, f.y), make_float2(f.z, f.w)};
+            }
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+          if (lane == 0) red[warp] = lsum;
+        }
+        if (st != L - 1 || !forward_only) {
+          fft<16, 1, true>(X, x);
+#pragma unroll
+          for (int n = 0; n < RL; ++n)
+            *reinterpret_cast<float4*>(sc + n * REGION) = make_float4(x[n].re.x, x[n].re.y, x[n].im.x, x[n].im.y);
+        }
+      }
+      __syncthreads();
+      if (st == L - 1) {
+        // the pattern has been read: the buffer takes the last slice's window again, or the next position's first
+        if (MODE != MODE_FORWARD) {
+          if (!p.loss_only) fetch_first(p.T + (size_t)(L - 1) * plane + oc);
+          else fetch_next_first();
+        }
+        if (MODE == MODE_FORWARD && L == 1) fetch_next_first();
+        if (forward_only) fetch_next_second();
+        state = (state & ~kFetched) | (window(state + 1) != kNoWindow ? kFetched : 0u);
+        fetch_origin(s);
+        fetch_commit();
+        if (MODE == MODE_FORWARD) break;
+        if (tid == 0) {
+          double acc = 0.0;
+#pragma unroll 1
+          for (int w = 0; w < NT / 32; ++w) acc += (double)red[w];
+          p.loss_part[s] = acc;
+        }
+        if (p.loss_only) break;
+      }
+      {   // ---------------- inverse pass B ----------------
+        float4* q = reinterpret_cast<float4*>(sb);
+        float2 x[32];
+        C2 X[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float4 f = q[i];
+          X[i] = {make_float2(f.x, f.y), make_float2(f.z, f.w)};
+        }
+        ifft32_dit(X, x);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) q[i] = make_float4(x[2 * i].x, x[2 * i].y, x[2 * i + 1].x, x[2 * i + 1].y);
+      }
+      __syncwarp();
+      a_in(v);
+      const int l = st < L - 1 ? st + 1 : 2 * L - 2 - st;
+      uint32_t f = 0;   // what this pass does
+      if (st < L - 1) {
+        f = kForward | kGoOn;
+        if (need_stash && (MODE == MODE_LOSS_GRAD || p.layer == l)) f |= kKeep;
+      } else {
+        if (MODE == MODE_LOSS_GRAD || (MODE == MODE_LAYER && l == p.layer)) f |= kGrad;
+        if (l > lowest || (l == 0 && MODE != MODE_LAYER && p.want_dprobe)) f |= kGoOn;
+        if (l > 0) f |= kPropagate;
+      }
+      const float2* T = p.T + (size_t)l * plane + oc;
+      if (word(f, kGoOn)) fetch_second(T);
+      float4* sl = stash + (MODE == MODE_LOSS_GRAD ? (size_t)l * (WW / 2) : 0);
+      fetch_commit();
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        C2 q[8];
+        fft<8, 1, true>(v[u], q);   // the incident wave of slice l, or chi_l
+        if (word(f, kGrad)) {
+          const int hs = half_slot(l, u);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            C2 e[4];
+            if (hs >= 0) {
+              tmem_load(tm + 32u * hs + 16u * i, e);
+            } else {
+#pragma unroll
+              for (int h = 0; h < 4; ++h) {
+                const float4 f = sl[(8 * u + 4 * i + h) * NT + tid];
+                e[h] = {make_float2(f.x, f.y), make_float2(f.z, f.w)};
+              }
+            }
+            gradient(s, l, u, i, oc, q + 4 * i, e);
+          }
+        }
+        if (CPLX && word(f, kKeep)) keep_half(l, u, sl, q);    // incident wave
+        fetch_wait<1>();
+        if (word(f, kForward)) transmit(kPlain, u, q);
+        else if (word(f, kGoOn)) transmit(kConj, u, q);        // conj(X_l) o chi_l
+        if (u == 0) {
+          if (word(f, kForward)) fetch_after(l);
+          else {
+            if (l > lowest) fetch_first(p.T + (size_t)(l - 1) * plane + oc);
+            else fetch_next_first();
+            fetch_commit();
+          }
+        }
+        if (!CPLX && word(f, kKeep)) keep_half(l, u, sl, q);   // exit wave
+        if (word(f, kForward | kPropagate)) {
+          fft<8, 1, false>(q, v[u]);
+        } else if (word(f, kGoOn)) {
+          // this CTA's probe-gradient partial: only this thread ever adds to these values, one position
+          // after another, so the order of the sums is fixed
+          float2* dp = p.dprobe_part + (size_t)blockIdx.x * WW + rc + CL * 2 * u;
+#pragma unroll
+          for (int h = 0; h < 8; ++h) {
+            const float2 a = make_float2(q[h].re.x, q[h].im.x), b = make_float2(q[h].re.y, q[h].im.y);
+            float2* d = dp + RL * h * W;
+            if (!word(state, kSummed)) {
+              d[0] = a;
+              d[CL] = b;
+            } else {
+              atomicAdd(d, a);
+              atomicAdd(d + CL, b);
+            }
+          }
+        }
+      }
+      if constexpr (kStash) tc::tmem_wait_st();
+      if (!word(f, kForward) && l == 0 && word(f, kGoOn)) state |= kSummed;
+      if (!word(f, kForward) && (l == 0 || !word(f, kGoOn))) {
+        fetch_next_second();
+        fetch_commit();
+        break;
+      }
+      a_out(v);
+    }
+  }
+
+  // a CTA whose every position was skipped still owns a (zero) probe partial
+  if ((MODE == MODE_LOSS_GRAD || MODE == MODE_PROBE) && p.want_dprobe && !(state & kSummed)) {
+    float2* dp = p.dprobe_part + (size_t)blockIdx.x * WW;
+    for (size_t i = tid; i < WW; i += NT) dp[i] = make_float2(0.f, 0.f);
+  }
+  if constexpr (kStash) {
     tc::fence_before();
     __syncthreads();
     if (tid < 32) {
@@ -487,20 +970,33 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
 // ----------------------------------------------------------------------------
 // launch helpers
 // ----------------------------------------------------------------------------
+template <int W, int MODE, bool CPLX>
+struct Kernel;
+template <int MODE, bool CPLX>
+struct Kernel<64, MODE, CPLX> {
+  static constexpr int NT = Geo<64>::NT;
+  static constexpr size_t SMEM = position_smem_bytes<64>();
+  static auto fn() { return position_kernel<64, MODE, CPLX>; }
+};
+template <int MODE, bool CPLX>
+struct Kernel<128, MODE, CPLX> {
+  static constexpr int NT = w128::NT;
+  static constexpr size_t SMEM = w128::SMEM;
+  static auto fn() { return position_kernel_128<MODE, CPLX>; }
+};
 
 template <int W, int MODE, bool CPLX>
 static cudaError_t launch_one(const PosParams& p, int grid, cudaStream_t st) {
-  const size_t smem = position_smem_bytes<W>();
+  using K = Kernel<W, MODE, CPLX>;
   static bool attr_done[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 64 && !attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(position_kernel<W, MODE, CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(K::fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::SMEM);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  position_kernel<W, MODE, CPLX><<<grid, 4 * W, smem, st>>>(p);
+  K::fn()<<<grid, K::NT, K::SMEM, st>>>(p);
   return cudaGetLastError();
 }
 
@@ -532,16 +1028,12 @@ cudaError_t launch_position_kernel(int win, int mode, const PosParams& p, int gr
 }
 
 // CTAs of the fused kernel that fit on one SM (same for every mode of a window size).
-static int position_ctas_per_sm(int win) {
+template <int W>
+static int position_ctas_per_sm() {
+  using K = Kernel<W, MODE_LOSS_GRAD, false>;
   int n = 0;
-  const size_t smem = win == 64 ? position_smem_bytes<64>() : position_smem_bytes<128>();
-  if (win == 64) {
-    cudaFuncSetAttribute(position_kernel<64, MODE_LOSS_GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, position_kernel<64, MODE_LOSS_GRAD>, 4 * 64, smem);
-  } else {
-    cudaFuncSetAttribute(position_kernel<128, MODE_LOSS_GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, position_kernel<128, MODE_LOSS_GRAD>, 4 * 128, smem);
-  }
+  cudaFuncSetAttribute(K::fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::SMEM);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, K::fn(), K::NT, K::SMEM);
   return n < 1 ? 1 : n;
 }
 
@@ -552,7 +1044,7 @@ int position_slots(int win) {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms * position_ctas_per_sm(win);
+  return sms * (win == 64 ? position_ctas_per_sm<64>() : position_ctas_per_sm<128>());
 }
 
 }  // namespace msp

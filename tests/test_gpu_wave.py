@@ -1,0 +1,120 @@
+"""The W = 128 kernel where its schedule changes (slices in tensor memory, windows fetched ahead, skipped
+positions, CTAs with one, two and three positions) and the far-field residual on operands that are not finite.
+
+Every position uses one of a few windows, so the oracle needs one evaluation per window.  The state is far from
+the data (kappa ~ 1), where the FP32 forward's rounding is not amplified: the bar is the 1e-5 of
+tests/test_gpu_parity.py."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import msp_oracle as O
+from workloads import synth
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def msp():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2205_03902_gb300 import msp
+    return msp
+
+
+def rel(a, b):
+    a, b = np.asarray(a), np.asarray(b)
+    return float(np.linalg.norm((a - b).ravel()) / max(np.linalg.norm(b.ravel()), 1e-300))
+
+
+def dev(a, dtype):
+    return torch.from_numpy(np.ascontiguousarray(a.astype(dtype))).cuda()
+
+
+class Problem:
+    def __init__(self, win, L, windows, obj, cplx=False, seed=3):
+        ny, nx = obj
+        rng = np.random.default_rng([seed, win, L])
+        self.gd = dict(n_slices=L, obj_ny=ny, obj_nx=nx, win=win, n_pos=0, wavelength_A=0.0698, sigma=1.54e-3, dz_A=2.0,
+                       pixel_A=0.15)
+        self.V = (300.0 * rng.standard_normal((L, ny, nx))).astype(np.float32).astype(np.float64)
+        self.T = None
+        if cplx:
+            t = (1 + 0.1 * rng.standard_normal((L, ny, nx))) * np.exp(1j * self.gd["sigma"] * self.V)
+            self.T = t.astype(np.complex64).astype(np.complex128)
+        p = synth.probe(synth.C2 if win == 128 else synth.C1, norm2=50.0)[:win, :win]
+        self.probe = p.astype(np.complex64).astype(np.complex128)
+        self.windows = np.asarray(windows, dtype=np.int32)
+        self.I = rng.poisson(3.0, size=(len(windows), win, win)).astype(np.float64)
+        kw = dict(T=self.T) if cplx else dict(V=self.V)
+        self.ref = [O.loss_grad(self.gd, self.probe, self.windows[k:k + 1], self.I[k:k + 1], **kw) for k in range(len(windows))]
+
+    def run(self, msp, order, bad=()):
+        """order: the window of each position; bad: positions whose window lies outside the object."""
+        pos, I = self.windows[order].copy(), self.I[order]
+        for b in bad:
+            pos[b] = (-1, 0) if b % 2 else (0, self.gd["obj_nx"])
+        g = msp.geometry(**{**self.gd, "n_pos": len(order)},
+                         param=msp.MSP_PARAM_POTENTIAL if self.T is None else msp.MSP_PARAM_TRANSMISSION)
+        V = dev(self.V, np.float32) if self.T is None else dev(self.T, np.complex64)
+        args = g, dev(self.probe, np.complex64), V, dev(pos, np.int32), dev(I, np.float32)
+        return args, msp.loss_grad(*args), [k for b, k in enumerate(order) if b not in bad]
+
+    def expect(self, good):
+        n = np.bincount(good, minlength=len(self.windows))
+        key = "dV" if self.T is None else "dX"
+        return (sum(c * r["loss"] for c, r in zip(n, self.ref)), sum(c * r[key] for c, r in zip(n, self.ref)),
+                sum(c * r["dprobe"] for c, r in zip(n, self.ref)))
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("L", [1, 2, 3, 4, 6])
+def test_slices_in_tensor_memory_and_in_the_stash(msp, L, cplx):
+    q = Problem(128, L, [(0, 0), (5, 3), (1, 12)], (133, 141), cplx)
+    _, (loss, dV, dp), good = q.run(msp, np.arange(7) % 3)
+    el, eV, ep = q.expect(good)
+    assert abs(float(loss) / el - 1) < TOL and rel(dV.cpu(), eV) < TOL and rel(dp.cpu(), ep) < TOL
+
+
+@pytest.mark.parametrize("L", [1, 3])
+def test_positions_of_a_cta_skipped_first_last_and_in_a_row(msp, L):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    q = Problem(128, L, [(0, 0), (5, 3), (1, 12), (4, 8)], (133, 141))
+    S = 3 * sms + 2
+    # CTA 0: its first skipped; 1: the second; 2: the last; 3: first and second; 4: all three; 5: none
+    bad = [0, 1 + sms, 2 + 2 * sms, 3, 3 + sms, 4, 4 + sms, 4 + 2 * sms]
+    args, (loss, dV, dp), good = q.run(msp, np.arange(S) % 4, bad)
+    el, eV, ep = q.expect(good)
+    assert abs(float(loss) / el - 1) < TOL and rel(dV.cpu(), eV) < TOL and rel(dp.cpu(), ep) < TOL
+    g, probe, V, pos, I = args
+    out = msp.forward(g, probe, V, pos).cpu().numpy()
+    only = msp.loss_grad(g, probe, V, pos, I, want_dV=False, want_dprobe=False)[0]
+    assert float(only) == float(loss)
+    ref = O.forward(q.gd, q.probe, q.windows, V=q.V)
+    for s in (1, 2, 5, sms, 2 * sms + 3, 3 * sms + 1):
+        assert rel(out[s], ref[s % 4]) < TOL
+    for b in bad:
+        assert not out[b].any()
+
+
+@pytest.mark.parametrize("win", [64, 128])
+@pytest.mark.parametrize("value", [np.inf, np.nan, -1.0, 0.0, 1e-42, 3e38])
+def test_residual_of_one_unusual_intensity(msp, win, value):
+    """One count replaced: the loss and the gradient follow sqrt and the quotient as IEEE arithmetic gives them."""
+    q = Problem(win, 1, [(0, 0), (2, 3)], (win + 5, win + 7))
+    k = (1, 3, 7)
+    q.I[k] = value
+    if np.isfinite(value) and value >= 0:
+        q.ref = [O.loss_grad(q.gd, q.probe, q.windows[j:j + 1], q.I[j:j + 1], V=q.V) for j in range(2)]
+        _, (loss, dV, dp), good = q.run(msp, np.arange(2))
+        el, eV, ep = q.expect(good)
+        assert abs(float(loss) / el - 1) < TOL and rel(dV.cpu(), eV) < TOL and rel(dp.cpu(), ep) < TOL
+    else:
+        _, (loss, dV, _), _ = q.run(msp, np.arange(2))
+        assert np.isinf(float(loss)) if value == np.inf else np.isnan(float(loss))
+        dV = dV.cpu().numpy()[0]
+        assert not np.isfinite(dV[2:2 + win, 3:3 + win]).any()      # the window of the pattern
+        assert np.isfinite(dV[0:2, 0:win]).all()                     # rows that only the other window covers
