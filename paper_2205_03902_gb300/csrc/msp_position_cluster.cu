@@ -222,17 +222,7 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(512, 1) position_clu
 #pragma unroll
             for (int m = 0; m < N1; ++m) out[(size_t)(j + T * m) * W] = fmaf(v[m].x, v[m].x, v[m].y * v[m].y);
           } else {
-#pragma unroll
-            for (int m = 0; m < N1; ++m) {
-              const float a2 = fmaf(v[m].x, v[m].x, v[m].y * v[m].y);
-              const float a = sqrtf(a2);
-              const float rt = sqrtf(im[m]);
-              const float d = rt - a;
-              lsum = fmaf(d, d, lsum);
-              // below the threshold the fraction is 0, so R = Psi (f = 1); a2 > zthr2 >= 0 implies a > 0
-              const float f = (a2 > zthr2) ? (1.f - rt / a) : 1.f;
-              v[m] = make_float2(v[m].x * f, v[m].y * f);
-            }
+            residual(v, im, zthr2, lsum);
             if (!p.loss_only) {
               line_fft<W, true, RegisterTwiddles<W, T>, T>(v, tw, xb, j);
 #pragma unroll
