@@ -89,7 +89,7 @@ template <bool CPLX, bool ILLUM, int LG>
 __device__ __forceinline__ void gather_tile(const float* __restrict__ src0, const float* __restrict__ src1,
                                             int nl_src, const int2* __restrict__ pos, int S, int W, int Ny, int Nx,
                                             float* __restrict__ out0, float* __restrict__ out1,
-                                            double* __restrict__ blockmax, int bx, int by, int l_first, int n_l,
+                                            float* __restrict__ blockmax, int bx, int by, int l_first, int n_l,
                                             int gx) {
   static_assert(!ILLUM || LG == 1, "the illumination channel is gathered for one slice");
   using Val = typename std::conditional<CPLX, float2, float>::type;
@@ -218,7 +218,7 @@ __device__ __forceinline__ void gather_tile(const float* __restrict__ src0, cons
     if (tid == 0) {
       float b = 0.f;
       for (int i = 0; i < 8; ++i) b = fmaxf(b, wmax[i]);
-      blockmax[by * gx + bx] = (double)b;
+      blockmax[by * gx + bx] = b;
     }
   }
 }
@@ -227,7 +227,8 @@ template <bool CPLX, bool ILLUM>
 __global__ void __launch_bounds__(256) gather_kernel(const float* __restrict__ src0, const float* __restrict__ src1,
                                                      int nl_src, const int2* __restrict__ pos, int S, int W,
                                                      int Ny, int Nx, float* __restrict__ out0,
-                                                     float* __restrict__ out1, double* __restrict__ blockmax) {
+                                                     float* __restrict__ out1, float* __restrict__ blockmax) {
+  wait_for_predecessor();
   gather_tile<CPLX, ILLUM, 1>(src0, src1, nl_src, pos, S, W, Ny, Nx, out0, out1, blockmax, blockIdx.x, blockIdx.y,
                               blockIdx.z, 1, gridDim.x);
 }
@@ -235,7 +236,8 @@ __global__ void __launch_bounds__(256) gather_kernel(const float* __restrict__ s
 // Per 32 x 8 object tile, the maximum of `map` (the gather's tiles and block-maximum layout):
 // the illumination maximum when the fused kernel summed the illumination map itself.
 __global__ void __launch_bounds__(256) tile_max_kernel(const float* __restrict__ map, int Ny, int Nx,
-                                                       double* __restrict__ blockmax) {
+                                                       float* __restrict__ blockmax) {
+  wait_for_predecessor();
   __shared__ float wmax[8];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int px = blockIdx.x * kGatherTX + (tid % kGatherTX), py = blockIdx.y * kGatherTY + (tid / kGatherTX);
@@ -247,7 +249,7 @@ __global__ void __launch_bounds__(256) tile_max_kernel(const float* __restrict__
   if (tid == 0) {
     float b = 0.f;
     for (int i = 0; i < 8; ++i) b = fmaxf(b, wmax[i]);
-    blockmax[blockIdx.y * gridDim.x + blockIdx.x] = (double)b;
+    blockmax[blockIdx.y * gridDim.x + blockIdx.x] = b;
   }
 }
 
@@ -313,17 +315,32 @@ __global__ void __launch_bounds__(256) sum_blocks_kernel(const float* __restrict
   if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-// dprobe[i] = sum_b part[b][i] (FP64 accumulation, fixed order).  A block of 256 threads owns 32
-// consecutive probe values: warp g sums the partials b = g, g + 8, g + 16, ... (lane = value, so
-// every load is 256 contiguous bytes), all of them in flight at once, and the eight warp sums
-// are added in warp order.  512 blocks for W = 128 keep every SM loading.
+// dprobe[i] = sum_b part[b][i], fixed order.  A block of 256 threads owns 32 consecutive probe values: warp g
+// sums the partials b = g, g + 8, g + 16, ... (lane = value, so every load is 256 contiguous bytes), all of
+// them in flight at once, and the eight warp sums are added in warp order.  512 blocks for W = 128 keep
+// every SM loading.  The sums are compensated (Knuth's two-sum, the rounding errors summed beside the sum):
+// about 48 bits before the one rounding to FP32, the same results as FP64 sums, whose additions and
+// conversions at 1/64 of the FP32 rate took most of the time (64 partials of W = 64: 10.7 us).
 constexpr int kDprobeVals = 32;
-__device__ __forceinline__ void dprobe_block(const float2* __restrict__ part, int G, int WW, float2* __restrict__ out,
-                                             int blk) {
-  __shared__ double2 acc_w[8][kDprobeVals];
+struct Compensated {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float t = s + v, b = t - s;
+    e += (s - (t - b)) + (v - b);
+    s = t;
+  }
+  __device__ __forceinline__ void add(const Compensated& c) {
+    add(c.s);
+    e += c.e;
+  }
+  __device__ __forceinline__ float value() const { return e == e ? s + e : s; }   // e is NaN where s is not finite
+};
+// the sum of value blk kDprobeVals + lane, in the lanes of warp 0
+__device__ __forceinline__ float2 dprobe_sum(const float2* __restrict__ part, int G, int WW, int blk) {
+  __shared__ Compensated acc_w[8][kDprobeVals][2];
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int i = blk * kDprobeVals + lane;
-  double re = 0.0, im = 0.0;
+  Compensated re, im;
   if (i < WW) {
     // all of a warp's partials (up to 24 at once) in flight, then added in ascending order
     constexpr int kBatch = 24;
@@ -335,26 +352,26 @@ __device__ __forceinline__ void dprobe_block(const float2* __restrict__ part, in
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {
         const bool live = b0 + 8 * u < G;
-        re += live ? (double)v[u].x : 0.0;
-        im += live ? (double)v[u].y : 0.0;
+        re.add(live ? v[u].x : 0.f);
+        im.add(live ? v[u].y : 0.f);
       }
     }
   }
-  acc_w[g][lane] = make_double2(re, im);
+  acc_w[g][lane][0] = re;
+  acc_w[g][lane][1] = im;
   __syncthreads();
-  if (g == 0 && i < WW) {
-    double2 t = acc_w[0][lane];
-    for (int w = 1; w < 8; ++w) {
-      t.x += acc_w[w][lane].x;
-      t.y += acc_w[w][lane].y;
-    }
-    out[i] = make_float2((float)t.x, (float)t.y);
+  if (g != 0) return make_float2(0.f, 0.f);
+  for (int w = 1; w < 8; ++w) {
+    re.add(acc_w[w][lane][0]);
+    im.add(acc_w[w][lane][1]);
   }
+  return make_float2(re.value(), im.value());
 }
-
-__global__ void __launch_bounds__(256) dprobe_reduce_kernel(const float2* __restrict__ part, int G, int WW,
-                                                            float2* __restrict__ out) {
-  dprobe_block(part, G, WW, out, blockIdx.x);
+__device__ __forceinline__ void dprobe_block(const float2* __restrict__ part, int G, int WW, float2* __restrict__ out,
+                                             int blk) {
+  const float2 t = dprobe_sum(part, G, WW, blk);
+  const int i = blk * kDprobeVals + (int)threadIdx.x;
+  if (threadIdx.x < kDprobeVals && i < WW) out[i] = t;
 }
 
 // The loss: the sum of n FP64 values in reduce_kernel's order (1024 strided partial sums, then
@@ -393,6 +410,7 @@ __global__ void __launch_bounds__(256) loss_grad_finish_kernel(const float* __re
                                                                float2* __restrict__ dprobe, int n_dprobe,
                                                                const double* __restrict__ loss_part, int n_loss,
                                                                double* __restrict__ loss, double* __restrict__ loss2) {
+  wait_for_predecessor();
   const int b = blockIdx.x;
   if (b < n_gather) {
     // the tile (bx, by) of slices l0 .. l0 + LG - 1 (LG = kGatherSlices, two if complex)
@@ -407,22 +425,21 @@ __global__ void __launch_bounds__(256) loss_grad_finish_kernel(const float* __re
   }
 }
 
-// Step size of a layer step: mu = step, or 1 / (c W^2 max illumination) with c = 2 sigma^2
-// (potential mode) or c = prod_{m > l} max |o_m|^2 (scal[6], transmission mode).
-// Set-up of every pass in one launch.  Block 0 clears the error word, forms the squared
-// zero-rule threshold tau^2 ||p||^2 (fixed-order sums) and the propagator factor
-// h1 (as propagator_kernel); every block converts its share of the potentials into
-// transmissions exp(i sigma V) (potential mode; n = 0 in transmission mode).
+// Set-up of every pass in one launch, its parts side by side: block 0 clears the error word and forms the
+// squared zero-rule threshold tau^2 ||p||^2 (fixed-order sums); the next W / 32 blocks form the propagator
+// factor h1 (as propagator_kernel), one warp each, since FP64 issues one warp instruction in sixteen clocks of
+// an SM (all of it in block 0: 8.5 us per launch); the others convert the potentials into transmissions
+// exp(i sigma V) (potential mode; none in transmission mode).
 __global__ void __launch_bounds__(1024) prepare_kernel(const float2* __restrict__ probe, int W, double tau2,
                                                        double* __restrict__ zthr2, float2* __restrict__ h1,
                                                        double dzlam, double dq, int* __restrict__ err,
                                                        const float* __restrict__ V, float2* __restrict__ T, size_t n,
                                                        float sigma) {
+  wait_for_predecessor();
+  const int tid = threadIdx.x, nh = W / 32;
   if (blockIdx.x == 0) {
-    // the squared zero-rule threshold tau^2 sum |p|^2: FP32 partials per thread and warp, the
-    // 32 warp sums in FP64 in a fixed order (FP64 throughput is low; a threshold needs no more)
+    // FP32 partials per thread and warp, the 32 warp sums in FP64 (a threshold needs no more)
     __shared__ float wsum[32];
-    const int tid = threadIdx.x;
     float a = 0.f;
     for (int i = tid; i < W * W; i += 1024) {
       const float2 v = probe[i];
@@ -432,67 +449,33 @@ __global__ void __launch_bounds__(1024) prepare_kernel(const float2* __restrict_
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if ((tid & 31) == 0) wsum[tid >> 5] = a;
     __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int i = 0; i < 32; ++i) t += (double)wsum[i];
-      zthr2[0] = tau2 * t;
-      err[0] = 0;
+    if (tid < 32) {
+      double t = (double)wsum[tid];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (tid == 0) {
+        zthr2[0] = tau2 * t;
+        err[0] = 0;
+      }
     }
-    for (int k = tid; k < W; k += 1024) {
-      const double q = (double)(k < W / 2 ? k : k - W) * dq;
-      double t = dzlam * q * q;   // phase / pi
-      t = t - 2.0 * floor(t * 0.5);
-      double sn, cs;
-      sincospi(t, &sn, &cs);
-      h1[k] = make_float2((float)(cs / W), (float)(-sn / W));
-    }
+    return;
   }
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+  if (blockIdx.x <= nh) {
+    if (tid >= 32) return;
+    const int k = 32 * (blockIdx.x - 1) + tid;
+    const double q = (double)(k < W / 2 ? k : k - W) * dq;
+    double t = dzlam * q * q;   // phase / pi
+    t = t - 2.0 * floor(t * 0.5);
+    double sn, cs;
+    sincospi(t, &sn, &cs);
+    h1[k] = make_float2((float)(cs / W), (float)(-sn / W));
+    return;
+  }
+  const size_t stride = (size_t)(gridDim.x - 1 - nh) * blockDim.x;
+  for (size_t i = (blockIdx.x - 1 - nh) * (size_t)blockDim.x + tid; i < n; i += stride) {
     float sn, cs;
     sincosf(sigma * V[i], &sn, &cs);
     T[i] = make_float2(cs, sn);
-  }
-}
-
-// End of a layer step's reductions in one launch, each in a fixed order (strided partials per
-// thread, a butterfly within each warp, the 32 warp values in order): the illumination
-// maximum (scal[2]) from the gather's per-tile maxima, the loss (scal[0], loss_out) from the
-// per-position partials, and the step mu (scal[1], mu_out) as layer_mu_kernel forms it.
-__global__ void __launch_bounds__(1024) layer_finish_kernel(const double* __restrict__ blockmax, int nblk,
-                                                            const double* __restrict__ loss_part, int nloss,
-                                                            double step, double c_w2, int cplx, double* scal,
-                                                            double* mu_out, double* loss_out) {
-  __shared__ double wm[32], ws[32];
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  double m = 0.0, a = 0.0;
-  for (int i = tid; i < nblk; i += 1024) m = fmax(m, blockmax[i]);
-  for (int i = tid; i < nloss; i += 1024) a += loss_part[i];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-  }
-  if (lane == 0) {
-    wm[w] = m;
-    ws[w] = a;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    double illum = 0.0, loss = 0.0;
-    for (int i = 0; i < 32; ++i) {
-      illum = fmax(illum, wm[i]);
-      loss += ws[i];
-    }
-    scal[2] = illum;
-    scal[0] = loss;
-    if (loss_out) loss_out[0] = loss;
-    double mu = step;
-    if (!(step > 0.0)) {
-      const double mm = illum * (cplx ? scal[6] : 1.0);
-      mu = (mm > 0.0) ? 1.0 / (c_w2 * mm) : 0.0;
-    }
-    scal[1] = mu;
-    if (mu_out) mu_out[0] = mu;
   }
 }
 
@@ -506,11 +489,70 @@ __global__ void layer_mu_kernel(double* scal, double step, double two_sig2_w2, d
   if (mu_out) mu_out[0] = mu;
 }
 
-__global__ void layer_update_kernel(float* __restrict__ V, const float* __restrict__ dV, size_t n,
-                                    const double* __restrict__ scal) {
-  const double mu = scal[1];
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+// End of a layer step in one launch: the last block sums the loss (loss_block's order), every other block
+// forms the step size from the gather's per-tile illumination maxima (each the same, mu = step or
+// 1 / (c W^2 max illumination) with c = 2 sigma^2 in potential mode and c = prod_{m > l} max |o_m|^2 (scal[6]) in
+// transmission mode) and updates its share of the slice.  A launch of its own for the reductions took 9 us.
+__global__ void __launch_bounds__(256) layer_update_kernel(float* __restrict__ V, const float* __restrict__ dV, size_t n,
+                                                           const float* __restrict__ tilemax, int ntiles,
+                                                           const double* __restrict__ loss_part, int nloss, double step,
+                                                           double c_w2, int cplx, double* scal, double* mu_out,
+                                                           double* loss_out) {
+  wait_for_predecessor();
+  if (blockIdx.x == gridDim.x - 1) {
+    loss_block(loss_part, nloss, scal, loss_out);
+    return;
+  }
+  __shared__ float wm[8];
+  __shared__ double s_mu;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  float m = 0.f;
+  for (int i = tid; i < ntiles; i += 256) m = fmaxf(m, tilemax[i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) wm[w] = m;
+  __syncthreads();
+  if (tid == 0) {
+    for (int i = 1; i < 8; ++i) m = fmaxf(m, wm[i]);
+    double mu = step;
+    if (!(step > 0.0)) {
+      const double mm = (double)m * (cplx ? scal[6] : 1.0);
+      mu = (mm > 0.0) ? 1.0 / (c_w2 * mm) : 0.0;
+    }
+    s_mu = mu;
+    if (blockIdx.x == 0) {
+      scal[2] = (double)m;
+      scal[1] = mu;
+      if (mu_out) mu_out[0] = mu;
+    }
+  }
+  __syncthreads();
+  const double mu = s_mu;
+  for (size_t i = blockIdx.x * (size_t)256 + tid; i < n; i += (size_t)(gridDim.x - 1) * 256)
     V[i] = (float)((double)V[i] - mu * (double)dV[i]);
+}
+
+// End of a probe step in one launch: block b sums the probe-gradient partials of its values and, without the
+// normalisation, takes the step p <- p - mu dprobe on them; the last block sums the loss.
+__global__ void __launch_bounds__(256) probe_finish_kernel(const float2* __restrict__ part, int G, int WW,
+                                                           float2* __restrict__ sum, float2* __restrict__ probe, double mu,
+                                                           const double* __restrict__ loss_part, int nloss, double* scal,
+                                                           double* mu_out, double* loss_out) {
+  wait_for_predecessor();
+  if (blockIdx.x == gridDim.x - 1) {
+    loss_block(loss_part, nloss, scal, loss_out);
+    if (threadIdx.x == 0 && mu_out) mu_out[0] = mu;
+    return;
+  }
+  const float2 g = dprobe_sum(part, G, WW, blockIdx.x);
+  const int i = blockIdx.x * kDprobeVals + (int)threadIdx.x;
+  if (threadIdx.x >= kDprobeVals || i >= WW) return;
+  if (probe) {
+    const float2 p = probe[i];
+    probe[i] = make_float2((float)((double)p.x - mu * (double)g.x), (float)((double)p.y - mu * (double)g.y));
+  } else {
+    sum[i] = g;
+  }
 }
 
 // Probe step p <- p - mu dprobe, optionally rescaled so that W^2 ||p||^2 = mean pattern sum.
@@ -752,11 +794,10 @@ static msp_status prepare(const msp_geometry* g, const float* probe, const float
   const int W = g->win;
   const bool pot = g->param != MSP_PARAM_TRANSMISSION;   // transmission mode uses the caller's slices as given
   const size_t n = pot ? (size_t)g->n_slices * g->obj_ny * g->obj_nx : 0;
-  const int blocks = (int)std::max<size_t>(1, std::min<size_t>((n + 1023) / 1024, (size_t)c.dev.sms * 4));
-  prepare_kernel<<<blocks, 1024, 0, c.st>>>((const float2*)probe, W, kZeroRuleTau * kZeroRuleTau, c.ws.scal + 5,
-                                            c.ws.h1, g->dz_A * g->wavelength_A, 1.0 / ((double)W * g->pixel_A),
-                                            c.ws.err, V, c.ws.T, n, (float)g->sigma);
-  MSP_CK(cudaGetLastError());
+  const int blocks = 1 + W / 32 + (int)std::min<size_t>((n + 1023) / 1024, (size_t)c.dev.sms * 4);
+  MSP_CK(launch_following(prepare_kernel, dim3(blocks), dim3(1024), 0, c.st, (const float2*)probe, W,
+                          kZeroRuleTau * kZeroRuleTau, c.ws.scal + 5, c.ws.h1, g->dz_A * g->wavelength_A,
+                          1.0 / ((double)W * g->pixel_A), c.ws.err, V, c.ws.T, n, (float)g->sigma));
   counted();
   return MSP_OK;
 }
@@ -927,17 +968,10 @@ msp_status msp_loss_grad(const msp_geometry* g, const float* probe, const float*
   const int n_gather = (dV && !l2_reduce) ? gx * gy * ((g->n_slices + lg - 1) / lg) : 0;
   const int n_dprobe = dprobe ? (int)((WW + kDprobeVals - 1) / kDprobeVals) : 0;
   const int nblk = n_gather + n_dprobe + 1;
-  if (p.cplx)
-    loss_grad_finish_kernel<true><<<nblk, 256, 0, c.st>>>(
-        c.ws.wgrad, (const int2*)pos, g->n_pos, W, g->n_slices, g->obj_ny, g->obj_nx, gx, gy, dV, n_gather,
-        c.ws.dprobe_part, c.parts, (float2*)dprobe, n_dprobe, c.ws.loss_part, g->n_pos * loss_slots(g), c.ws.scal,
-        loss);
-  else
-    loss_grad_finish_kernel<false><<<nblk, 256, 0, c.st>>>(
-        c.ws.wgrad, (const int2*)pos, g->n_pos, W, g->n_slices, g->obj_ny, g->obj_nx, gx, gy, dV, n_gather,
-        c.ws.dprobe_part, c.parts, (float2*)dprobe, n_dprobe, c.ws.loss_part, g->n_pos * loss_slots(g), c.ws.scal,
-        loss);
-  MSP_CK(cudaGetLastError());
+  MSP_CK(launch_following(p.cplx ? loss_grad_finish_kernel<true> : loss_grad_finish_kernel<false>, dim3(nblk), dim3(256), 0,
+                          c.st, c.ws.wgrad, (const int2*)pos, g->n_pos, W, g->n_slices, g->obj_ny, g->obj_nx, gx, gy, dV,
+                          n_gather, c.ws.dprobe_part, c.parts, (float2*)dprobe, n_dprobe, c.ws.loss_part,
+                          g->n_pos * loss_slots(g), c.ws.scal, loss));
   counted();
   return MSP_OK;
 }
@@ -983,15 +1017,13 @@ msp_status msp_layer_step(const msp_geometry* g, const float* probe, float* V, c
     p.illumred = c.ws.map1;
   }
   MSP_TRY(run_position(g, MODE_LAYER, p, c));
+  float* tilemax = (float*)c.ws.red;
   if (l2_reduce)
-    tile_max_kernel<<<grid, 256, 0, c.st>>>(c.ws.map1, g->obj_ny, g->obj_nx, c.ws.red);
-  else if (p.cplx)
-    gather_kernel<true, true><<<grid, 256, 0, c.st>>>(c.ws.wgrad, c.ws.willum, 1, (const int2*)pos, g->n_pos, W,
-                                                      g->obj_ny, g->obj_nx, c.ws.map0, c.ws.map1, c.ws.red);
+    MSP_CK(launch_following(tile_max_kernel, grid, dim3(256), 0, c.st, c.ws.map1, g->obj_ny, g->obj_nx, tilemax));
   else
-    gather_kernel<false, true><<<grid, 256, 0, c.st>>>(c.ws.wgrad, c.ws.willum, 1, (const int2*)pos, g->n_pos, W,
-                                                       g->obj_ny, g->obj_nx, c.ws.map0, c.ws.map1, c.ws.red);
-  MSP_CK(cudaGetLastError());
+    MSP_CK(launch_following(p.cplx ? gather_kernel<true, true> : gather_kernel<false, true>, grid, dim3(256), 0, c.st,
+                            c.ws.wgrad, c.ws.willum, 1, (const int2*)pos, g->n_pos, W, g->obj_ny, g->obj_nx, c.ws.map0,
+                            c.ws.map1, tilemax));
   counted();
   if (p.cplx) {
     later_slices_gain_kernel<<<1, 1024, 0, c.st>>>((const float2*)V, g->n_slices, plane, layer, c.ws.scal + 6);
@@ -1000,15 +1032,12 @@ msp_status msp_layer_step(const msp_geometry* g, const float* probe, float* V, c
   }
   // potential mode: mu = 1 / (2 sigma^2 W^2 max illum); transmission: 1 / (W^2 max illum prod max|o_m|^2)
   const double c_w2 = (p.cplx ? 1.0 : 2.0 * g->sigma * g->sigma) * (double)W * (double)W;
-  layer_finish_kernel<<<1, 1024, 0, c.st>>>(c.ws.red, nblk, c.ws.loss_part, g->n_pos * loss_slots(g), step, c_w2,
-                                            p.cplx, c.ws.scal, mu_out, loss_before);
-  MSP_CK(cudaGetLastError());
-  counted();
   // V_l (or the complex o_l, as interleaved floats) -= mu * gradient map
   const size_t nupd = plane * (p.cplx ? 2 : 1);
-  const int blocks = (int)std::min<size_t>((nupd + 255) / 256, (size_t)c.dev.sms * 8);
-  layer_update_kernel<<<blocks, 256, 0, c.st>>>(V + (size_t)layer * nupd, c.ws.map0, nupd, c.ws.scal);
-  MSP_CK(cudaGetLastError());
+  const int blocks = 1 + (int)std::min<size_t>((nupd + 255) / 256, (size_t)c.dev.sms);
+  MSP_CK(launch_following(layer_update_kernel, dim3(blocks), dim3(256), 0, c.st, V + (size_t)layer * nupd, c.ws.map0, nupd,
+                          tilemax, nblk, c.ws.loss_part, g->n_pos * loss_slots(g), step, c_w2, p.cplx, c.ws.scal, mu_out,
+                          loss_before));
   counted();
   return MSP_OK;
 }
@@ -1035,17 +1064,19 @@ msp_status msp_probe_step(const msp_geometry* g, float* probe, const float* V, c
   const double mu = (step > 0.0) ? step : (S > 0 ? 1.0 / ((double)S * (double)WW) : 0.0);
   if (S == 0) {
     MSP_CK(cudaMemsetAsync(c.ws.dprobe_sum, 0, WW * sizeof(float2), c.st));
+    MSP_TRY(reduce_loss(g, c, loss_before));
   } else {
     PosParams p = base_params(g, probe, V, pos, c);
     p.I_meas = I_meas;
     p.want_dprobe = 1;
     MSP_TRY(run_position(g, MODE_PROBE, p, c));
-    dprobe_reduce_kernel<<<(int)((WW + kDprobeVals - 1) / kDprobeVals), 256, 0, c.st>>>(c.ws.dprobe_part, c.parts, (int)WW,
-                                                                   c.ws.dprobe_sum);
-    MSP_CK(cudaGetLastError());
-  counted();
+    const int nb = (int)((WW + kDprobeVals - 1) / kDprobeVals);
+    MSP_CK(launch_following(probe_finish_kernel, dim3(nb + 1), dim3(256), 0, c.st, c.ws.dprobe_part, c.parts, (int)WW,
+                            c.ws.dprobe_sum, normalize ? nullptr : (float2*)probe, mu, c.ws.loss_part,
+                            g->n_pos * loss_slots(g), c.ws.scal, normalize ? nullptr : mu_out, loss_before));
+    counted();
+    if (!normalize) return MSP_OK;
   }
-  MSP_TRY(reduce_loss(g, c, loss_before));
   if (normalize && S > 0) {
     const int nb = 1024;
     sum_blocks_kernel<<<nb, 256, 0, c.st>>>(I_meas, (size_t)S * WW, c.ws.red);

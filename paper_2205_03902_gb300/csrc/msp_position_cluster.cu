@@ -74,12 +74,8 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(512, 1) position_clu
   const size_t plane = (size_t)p.Ny * p.Nx;
   float2* xb = sm + RW * W + grp * T * XS;
 
-  if (tid < N1 * T) {   // evaluated in double, rounded once
-    const int k1 = tid / T, jj = tid % T;
-    double sn, cs;
-    sincospi(2.0 * (double)((jj * k1) % W) / (double)W, &sn, &cs);
-    s_tw[tid] = make_float2((float)cs, (float)-sn);
-  }
+  if (tid < N1 * T) s_tw[tid] = twiddle<W>(((tid / T) * (tid % T)) % W);
+  wait_for_predecessor();
   if (tid < W) s_h1[tid] = p.h1[tid];
   __syncthreads();
   const RegisterTwiddles<W, T> tw(s_tw, j);
@@ -358,8 +354,8 @@ static cudaError_t launch_cluster_one(const PosParams& p, int clusters, cudaStre
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  position_cluster_kernel<MODE, CPLX><<<clusters * c256::CL, c256::NT, c256::SMEM, st>>>(p);
-  return cudaGetLastError();
+  void (*kernel)(const PosParams) = position_cluster_kernel<MODE, CPLX>;
+  return launch_following(kernel, dim3(clusters * c256::CL), dim3(c256::NT), c256::SMEM, st, p);
 }
 
 template <bool CPLX>
