@@ -248,10 +248,9 @@ def _arrays(g: Geometry, probe, V, pos, I=None, I_name="I_meas"):
 
 def forward(g: Geometry, probe, V, pos, out=None, ws=None, stream=None):
     """Far-field intensities [S][W][W] (msp_forward)."""
-    device = _arrays(g, probe, V, pos)
+    device = _arrays(g, probe, V, pos, out, "out")
     if out is None:
         out = torch.empty((g.n_pos, g.win, g.win), dtype=torch.float32, device=device)
-    _arrays(g, probe, V, pos, out, "out")
     ws = _ws(g, ws, device)
     _check(lib().msp_forward(ctypes.byref(g), _ptr(probe), _ptr(V), _ptr(pos), _ptr(out), ws.ptr(), ws.nbytes,
                              _stream(stream)), "msp_forward")
