@@ -38,6 +38,7 @@
 #include <type_traits>
 
 #include "msp.h"
+#include "msp_fft.cuh"
 #include "msp_kernels.cuh"
 
 namespace msp {
@@ -88,9 +89,6 @@ template <> __device__ __forceinline__ double2 from_d<double2>(double re, double
 struct dff {
   float h, l;
 };
-struct dfc {   // complex: re, im
-  dff re, im;
-};
 __device__ __forceinline__ dff two_sum(float a, float b) {
   const float s = a + b, bb = s - a;
   return {s, (a - (s - bb)) + (b - bb)};
@@ -132,18 +130,64 @@ __device__ __forceinline__ dff df_div(dff a, dff b) {   // a / b, b != 0
   return fast_two_sum(q0, r / b.h);
 }
 
-__device__ __forceinline__ dfc add(dfc a, dfc b) { return {df_add(a.re, b.re), df_add(a.im, b.im)}; }
-__device__ __forceinline__ dfc sub(dfc a, dfc b) { return {df_add(a.re, df_neg(b.re)), df_add(a.im, df_neg(b.im))}; }
-__device__ __forceinline__ dfc mul(dfc a, dfc b) {
-  return {df_add(df_mul(a.re, b.re), df_neg(df_mul(a.im, b.im))), df_add(df_mul(a.re, b.im), df_mul(a.im, b.re))};
+// Complex: the high and the low parts of (re, im) side by side, so that one packed instruction works on
+// both components: an operation on dfc is the operation above on each, rounding for rounding, in half the
+// instructions.  The kernels below run straight through several thousand of them, and waited for
+// instructions more than for anything else (4.3 of 9.5 stall cycles per issue before, W = 128).
+struct alignas(16) dfc {
+  float2 h, l;
+  __device__ __forceinline__ dff re() const { return {h.x, l.x}; }
+  __device__ __forceinline__ dff im() const { return {h.y, l.y}; }
+};
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ dfc fast_two_sum(float2 a, float2 b) {
+  const float2 s = add2(a, b);
+  return {s, sub2(b, sub2(s, a))};
 }
-__device__ __forceinline__ dfc mulc(dfc a, dfc b) {   // a * conj(b)
-  return {df_add(df_mul(a.re, b.re), df_mul(a.im, b.im)), df_add(df_mul(a.im, b.re), df_neg(df_mul(a.re, b.im)))};
+__device__ __forceinline__ dfc add(dfc a, dfc b) {
+  const float2 s = add2(a.h, b.h), bb = sub2(s, a.h);
+  const float2 e = add2(sub2(a.h, sub2(s, bb)), sub2(b.h, bb));
+  return fast_two_sum(s, add2(e, add2(a.l, b.l)));
 }
-__device__ __forceinline__ double2 widen(dfc a) { return make_double2(df_to(a.re), df_to(a.im)); }
-__device__ __forceinline__ float2 narrow(dfc a) { return make_float2((float)df_to(a.re), (float)df_to(a.im)); }
-template <> __device__ __forceinline__ dfc from_f2<dfc>(float2 a) { return {{a.x, 0.f}, {a.y, 0.f}}; }
-template <> __device__ __forceinline__ dfc from_d<dfc>(double re, double im) { return {df_from(re), df_from(im)}; }
+__device__ __forceinline__ dfc sub(dfc a, dfc b) {   // a + (-b)
+  const float2 s = sub2(a.h, b.h), bb = sub2(s, a.h);
+  const float2 e = sub2(sub2(a.h, sub2(s, bb)), add2(b.h, bb));
+  return fast_two_sum(s, add2(e, sub2(a.l, b.l)));
+}
+// a times the real y.h + y.l (both components of yh, yl the same)
+__device__ __forceinline__ dfc scale(dfc a, float2 yh, float2 yl) {
+  const float2 p = mul2(a.h, yh);
+  float2 e = fma2(a.h, yh, neg2(p));
+  e = fma2(a.h, yl, e);
+  e = fma2(a.l, yh, e);
+  return fast_two_sum(p, e);
+}
+__device__ __forceinline__ dfc times_i(dfc a) { return {make_float2(-a.h.y, a.h.x), make_float2(-a.l.y, a.l.x)}; }
+__device__ __forceinline__ dfc times_mi(dfc a) { return {make_float2(a.h.y, -a.h.x), make_float2(a.l.y, -a.l.x)}; }
+// a factor of complex products with each part twice, as the packed products take it
+struct alignas(16) dfw {
+  float2 reh, rel, imh, iml;
+};
+__device__ __forceinline__ dfw twice(dfc b) { return {both(b.h.x), both(b.l.x), both(b.h.y), both(b.l.y)}; }
+__device__ __forceinline__ dfc mul(dfc a, dfw b) { return add(scale(a, b.reh, b.rel), times_i(scale(a, b.imh, b.iml))); }
+__device__ __forceinline__ dfc mulc(dfc a, dfw b) {   // a * conj(b)
+  return add(scale(a, b.reh, b.rel), times_mi(scale(a, b.imh, b.iml)));
+}
+__device__ __forceinline__ dfc mul(dfc a, dfc b) { return mul(a, twice(b)); }
+__device__ __forceinline__ dfc mulc(dfc a, dfc b) { return mulc(a, twice(b)); }
+__device__ __forceinline__ double2 widen(dfc a) { return make_double2(df_to(a.re()), df_to(a.im())); }
+__device__ __forceinline__ float2 narrow(dfc a) { return make_float2((float)df_to(a.re()), (float)df_to(a.im())); }
+template <> __device__ __forceinline__ dfc from_f2<dfc>(float2 a) { return {a, make_float2(0.f, 0.f)}; }
+template <> __device__ __forceinline__ dfc from_d<dfc>(double re, double im) {
+  const dff r = df_from(re), i = df_from(im);
+  return {make_float2(r.h, i.h), make_float2(r.l, i.l)};
+}
+// the form in which a line transform keeps its twiddles
+template <typename C> struct Factor { using type = C; };
+template <> struct Factor<dfc> { using type = dfw; };
+template <typename C> __device__ __forceinline__ typename Factor<C>::type factor(C a) { return a; }
+template <> __device__ __forceinline__ dfw factor<dfc>(dfc a) { return twice(a); }
 
 __device__ __forceinline__ bool window_ok(int2 ps, int Ny, int Nx, int W) {
   return ps.x >= 0 && ps.y >= 0 && ps.x <= Ny - W && ps.y <= Nx - W;
@@ -155,11 +199,11 @@ __device__ __forceinline__ bool window_ok(int2 ps, int Ny, int Nx, int W) {
 // ---------------------------------------------------------------------------
 template <typename C> __device__ __forceinline__ C from_h(C h) { return h; }
 template <typename C> __device__ __forceinline__ C conj_(C a) { return mk<C>(a.x, -a.y); }
-template <> __device__ __forceinline__ dfc conj_<dfc>(dfc a) { return {a.re, df_neg(a.im)}; }
+template <> __device__ __forceinline__ dfc conj_<dfc>(dfc a) { return {make_float2(a.h.x, -a.h.y), make_float2(a.l.x, -a.l.y)}; }
 template <typename C> __device__ __forceinline__ C rot_mi(C a) { return mk<C>(a.y, -a.x); }   // a (-i)
-template <> __device__ __forceinline__ dfc rot_mi<dfc>(dfc a) { return {a.im, df_neg(a.re)}; }
+template <> __device__ __forceinline__ dfc rot_mi<dfc>(dfc a) { return times_mi(a); }
 template <typename C> __device__ __forceinline__ C neg_(C a) { return mk<C>(-a.x, -a.y); }
-template <> __device__ __forceinline__ dfc neg_<dfc>(dfc a) { return {df_neg(a.re), df_neg(a.im)}; }
+template <> __device__ __forceinline__ dfc neg_<dfc>(dfc a) { return {neg2(a.h), neg2(a.l)}; }
 
 // cos and sin of 2 pi k / 16, k = 0..3, as exact decimal expansions of the regular 16-gon
 constexpr double kCos16[4] = {1.0, 0.92387953251128675613, 0.70710678118654752440, 0.38268343236508977173};
@@ -182,7 +226,7 @@ template <> __device__ __forceinline__ float2 w16c<float2, 0>() { return make_fl
   template <> __device__ __forceinline__ dfc w16c<dfc, K>() {                                            \
     constexpr double c = cos16<K>(), sn = -sin16<K>();                                                    \
     constexpr float ch = (float)c, sh = (float)sn;                                                        \
-    return {{ch, (float)(c - (double)ch)}, {sh, (float)(sn - (double)sh)}};                               \
+    return {make_float2(ch, sh), make_float2((float)(c - (double)ch), (float)(sn - (double)sh))};         \
   }
 MSP_W16(1) MSP_W16(2) MSP_W16(3) MSP_W16(5) MSP_W16(6) MSP_W16(7) MSP_W16(9) MSP_W16(10) MSP_W16(11)
 MSP_W16(13) MSP_W16(14) MSP_W16(15)
@@ -224,7 +268,7 @@ __device__ __forceinline__ void dft_g(const C* x, C* X) {
 // N1-point DFTs for N1 = 32 (W = 256): two 16-point DFTs and one radix-2 combination with the
 // twiddles w_32^k = from the line's table (tw32[k] = w_W^(k W / 32)).
 template <typename C, int N1>
-__device__ __forceinline__ void dft_n1(const C* x, C* X, const C* __restrict__ tw32) {
+__device__ __forceinline__ void dft_n1(const C* x, C* X, const typename Factor<C>::type* __restrict__ tw32) {
   if constexpr (N1 <= 16) {
     dft_g<C, N1, 1>(x, X);
   } else {
@@ -258,7 +302,8 @@ struct LinesCfg {
 // step B the twiddles w_W^(j k1) (s_tw[k1 kT + j]), an exchange through the group's shared
 // buffer xb, step C N1/8 eight-point DFTs.
 template <typename C, int W>
-__device__ __forceinline__ void line_dft(C (&v)[W / kT], const C* __restrict__ s_tw, const C* __restrict__ s_t32,
+__device__ __forceinline__ void line_dft(C (&v)[W / kT], const typename Factor<C>::type* __restrict__ s_tw,
+                                         const typename Factor<C>::type* __restrict__ s_t32,
                                          C* xb, int j) {
   constexpr int N1 = W / kT, XS = N1 + 1, NC = N1 / kT;
   C y[N1];
@@ -287,10 +332,11 @@ __device__ __forceinline__ void line_dft(C (&v)[W / kT], const C* __restrict__ s
 // The twiddle tables of a CTA's line transforms: s_tw[k1 kT + j] = w_W^(j k1) and, for N1 = 32,
 // s_t32[k] = w_32^k, from wtab[k] = w_256^k.
 template <typename C, int W, int NT>
-__device__ __forceinline__ void load_twiddles(C* s_tw, C* s_t32, const C* __restrict__ wtab) {
+__device__ __forceinline__ void load_twiddles(typename Factor<C>::type* s_tw, typename Factor<C>::type* s_t32,
+                                              const C* __restrict__ wtab) {
   constexpr int N1 = W / kT, STEP = 256 / W;
-  for (int i = threadIdx.x; i < N1 * kT; i += NT) s_tw[i] = wtab[((i / kT) * (i % kT) * STEP) % 256];
-  if (N1 > 16 && threadIdx.x < 16) s_t32[threadIdx.x] = wtab[threadIdx.x * 8];
+  for (int i = threadIdx.x; i < N1 * kT; i += NT) s_tw[i] = factor<C>(wtab[((i / kT) * (i % kT) * STEP) % 256]);
+  if (N1 > 16 && threadIdx.x < 16) s_t32[threadIdx.x] = factor<C>(wtab[threadIdx.x * 8]);
 }
 
 // The column half of a Fresnel propagation of row-transformed waves: every column is
@@ -303,8 +349,8 @@ __global__ void __launch_bounds__(LinesCfg<C, W>::THREADS) cols_propagate_kernel
                                                                                 const H* __restrict__ h1) {
   using Cfg = LinesCfg<C, W>;
   constexpr int N1 = Cfg::N1, XS = Cfg::XS, LPC = Cfg::LPC;
-  __shared__ C s_tw[N1 * kT];
-  __shared__ C s_t32[16];
+  __shared__ typename Factor<C>::type s_tw[N1 * kT];
+  __shared__ typename Factor<C>::type s_t32[16];
   __shared__ C xbuf[LPC][kT * XS];
   load_twiddles<C, W, Cfg::THREADS>(s_tw, s_t32, wtab);
   __syncthreads();
@@ -408,8 +454,8 @@ __global__ void __launch_bounds__(LinesCfg<C, W>::THREADS) rows_transmit_kernel(
   using Cfg = LinesCfg<C, W>;
   constexpr int N1 = Cfg::N1, XS = Cfg::XS, LPC = Cfg::LPC;
   constexpr size_t WW = (size_t)W * W;
-  __shared__ C s_tw[N1 * kT];
-  __shared__ C s_t32[16];
+  __shared__ typename Factor<C>::type s_tw[N1 * kT];
+  __shared__ typename Factor<C>::type s_t32[16];
   __shared__ C xbuf[LPC][kT * XS];
   load_twiddles<C, W, Cfg::THREADS>(s_tw, s_t32, wtab);
   __syncthreads();
@@ -509,17 +555,17 @@ __device__ __forceinline__ float2 residual_value(double2 v, float I, double thr2
   return make_float2((float)(v.x * f), (float)(v.y * f));
 }
 __device__ __forceinline__ float2 residual_value(dfc v, float I, double thr2, double& acc) {
-  const dff a2 = df_add(df_mul(v.re, v.re), df_mul(v.im, v.im));
+  const dff re = v.re(), im = v.im(), a2 = df_add(df_mul(re, re), df_mul(im, im));
   const dff a = df_sqrt(a2), rt = df_sqrt(dff{I, 0.f});
   const double dd = df_to(df_add(rt, df_neg(a)));
   acc += dd * dd;
   const dff f = df_to(a2) > thr2 ? df_add(dff{1.f, 0.f}, df_neg(df_div(rt, a))) : dff{1.f, 0.f};
-  const dff rx = df_mul(v.re, f), ry = df_mul(v.im, f);
+  const dff rx = df_mul(re, f), ry = df_mul(im, f);
   return make_float2(rx.h + rx.l, ry.h + ry.l);
 }
 __device__ __forceinline__ float intensity_value(double2 v) { return (float)(v.x * v.x + v.y * v.y); }
 __device__ __forceinline__ float intensity_value(dfc v) {
-  const dff a2 = df_add(df_mul(v.re, v.re), df_mul(v.im, v.im));
+  const dff re = v.re(), im = v.im(), a2 = df_add(df_mul(re, re), df_mul(im, im));
   return a2.h + a2.l;
 }
 
@@ -537,8 +583,8 @@ __global__ void __launch_bounds__(LinesCfg<C, W>::THREADS) cols_farfield_kernel(
   using Cfg = LinesCfg<C, W>;
   constexpr int N1 = Cfg::N1, XS = Cfg::XS, LPC = Cfg::LPC, NT = Cfg::THREADS;
   constexpr size_t WW = (size_t)W * W;
-  __shared__ C s_tw[N1 * kT];
-  __shared__ C s_t32[16];
+  __shared__ typename Factor<C>::type s_tw[N1 * kT];
+  __shared__ typename Factor<C>::type s_t32[16];
   __shared__ float2 s_tw8[N1 * kT];
   __shared__ float2 s_t328[16];
   __shared__ C xbuf[LPC][kT * XS];
