@@ -322,19 +322,6 @@ __global__ void __launch_bounds__(256) sum_blocks_kernel(const float* __restrict
 // about 48 bits before the one rounding to FP32, the same results as FP64 sums, whose additions and
 // conversions at 1/64 of the FP32 rate took most of the time (64 partials of W = 64: 10.7 us).
 constexpr int kDprobeVals = 32;
-struct Compensated {
-  float s = 0.f, e = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float t = s + v, b = t - s;
-    e += (s - (t - b)) + (v - b);
-    s = t;
-  }
-  __device__ __forceinline__ void add(const Compensated& c) {
-    add(c.s);
-    e += c.e;
-  }
-  __device__ __forceinline__ float value() const { return e == e ? s + e : s; }   // e is NaN where s is not finite
-};
 // the sum of value blk kDprobeVals + lane, in the lanes of warp 0
 __device__ __forceinline__ float2 dprobe_sum(const float2* __restrict__ part, int G, int WW, int blk) {
   __shared__ Compensated acc_w[8][kDprobeVals][2];

@@ -60,6 +60,23 @@ inline cudaError_t launch_following(void (*kernel)(P...), dim3 grid, dim3 block,
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// A compensated FP32 sum (Knuth's two-sum, the rounding errors summed beside the sum): about 48 bits.
+struct Compensated {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float t = s + v, b = t - s;
+    e += (s - (t - b)) + (v - b);
+    s = t;
+  }
+  __device__ __forceinline__ void add(const Compensated& c) {
+    add(c.s);
+    e += c.e;
+  }
+  // e is NaN where s is not finite
+  __device__ __forceinline__ float value() const { return e == e ? s + e : s; }
+  __device__ __forceinline__ double wide() const { return e == e ? (double)s + (double)e : (double)s; }
+};
+
 // Workspace carve-up (all offsets 256-byte aligned).
 struct Workspace {
   int* err;

@@ -372,48 +372,9 @@ __global__ void __launch_bounds__(LinesCfg<C, W>::THREADS) cols_propagate_kernel
   for (int m = 0; m < N1; ++m) img[(size_t)(j + kT * m) * W + line] = conj_(v[m]);
 }
 
-// wtab[k] = exp(-2 pi i k / 256), evaluated in double, rounded (FP32) or split (double-float) once
-template <typename C>
-__global__ void wtab_kernel(C* __restrict__ wtab) {
-  const int k = threadIdx.x;
-  double sn, cs;
-  sincospi(2.0 * (double)k / 256.0, &sn, &cs);
-  wtab[k] = from_d<C>(cs, -sn);
-}
-
 // ---------------------------------------------------------------------------
 // element-wise kernels over a batch [nb][W][W]
 // ---------------------------------------------------------------------------
-
-// FP64 slice transmissions: exp(i sigma V) from the FP32 potentials, or the caller's complex
-// slices widened.
-template <typename C>
-__global__ void table64_kernel(const float* __restrict__ V, const float2* __restrict__ X, C* __restrict__ T, size_t n,
-                               double sigma) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    if (X) {
-      T[i] = from_f2<C>(X[i]);
-    } else {
-      double sn, cs;
-      sincos(sigma * (double)V[i], &sn, &cs);
-      T[i] = from_d<C>(cs, sn);
-    }
-  }
-}
-
-// h1(k) = exp(-i pi dz lambda q_k^2) / W in double (the propagator factor of the fast path
-// before its rounding to single).
-template <typename C>
-__global__ void h1_64_kernel(C* __restrict__ h1, int W, double dzlam, double dq) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= W) return;
-  const double q = (double)(k < W / 2 ? k : k - W) * dq;
-  double t = dzlam * q * q;
-  t = t - 2.0 * floor(t * 0.5);
-  double sn, cs;
-  sincospi(t, &sn, &cs);
-  h1[k] = from_d<C>(cs / W, -sn / W);
-}
 
 struct Batch {
   const int2* pos;     // positions of this batch (pos + b0)
@@ -729,32 +690,27 @@ __global__ void __launch_bounds__(LinesCfg<float2, W>::THREADS) rows_adjoint_ker
   }
 }
 
-// dp64[k] += sum_{b < nb} contrib[b][k], b ascending (FP64, fixed order); eight loads in flight
-// per thread, added in the same order.
-__global__ void dprobe_accumulate_kernel(const float2* __restrict__ contrib, int nb, int WW, double2* __restrict__ dp64,
-                                         int first) {
+// dp64[k] += sum_{b < nb} contrib[b][k], b ascending (fixed order), eight loads in flight per thread.  The sum over
+// a batch is compensated FP32 (about 48 bits), added to the FP64 sum once: FP64 additions and conversions of
+// every term took 56 us for 169 positions of W = 128.  Blocks of 64 threads spread the image over the SMs.
+__global__ void __launch_bounds__(64) dprobe_accumulate_kernel(const float2* __restrict__ contrib, int nb, int WW,
+                                                               double2* __restrict__ dp64, int first) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= WW) return;
-  double2 a = first ? make_double2(0.0, 0.0) : dp64[k];
-  int b = 0;
-  for (; b + 8 <= nb; b += 8) {
+  Compensated x, y;
+  for (int b = 0; b < nb; b += 8) {
     float2 v[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = contrib[(size_t)(b + u) * WW + k];
+    for (int u = 0; u < 8; ++u) v[u] = b + u < nb ? contrib[(size_t)(b + u) * WW + k] : make_float2(0.f, 0.f);
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      a.x += v[u].x;
-      a.y += v[u].y;
+      x.add(v[u].x);
+      y.add(v[u].y);
     }
   }
-  for (; b < nb; ++b) {
-    const float2 v = contrib[(size_t)b * WW + k];
-    a.x += v.x;
-    a.y += v.y;
-  }
-  dp64[k] = a;
+  const double2 a = first ? make_double2(0.0, 0.0) : dp64[k];
+  dp64[k] = make_double2(a.x + x.wide(), a.y + y.wide());
 }
-
 __global__ void dprobe_finish_kernel(const double2* __restrict__ dp64, int WW, float2* __restrict__ out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < WW) out[k] = narrow(dp64[k]);
@@ -763,6 +719,57 @@ __global__ void dprobe_finish_kernel(const double2* __restrict__ dp64, int WW, f
 __global__ void flag_windows_kernel(const int2* __restrict__ pos, int S, int Ny, int Nx, int W, int* err) {
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S; s += gridDim.x * blockDim.x)
     if (!window_ok(pos[s], Ny, Nx, W)) atomicMax(err, 1);
+}
+
+// Set-up of a pass in one launch, its parts side by side (they are FP64 chains of a few warps beside the table;
+// five launches, one after another, took 32 us at L = 4 on 233 x 224 pixels):
+//   blocks [0, nt)      T = exp(i sigma V) from the FP32 potentials, or the caller's complex slices widened
+//   the next W / 32     h1(k) = exp(-i pi dz lambda q_k^2) / W in double (the propagator factor of the fast path
+//                       before its rounding to single), one warp each
+//   the next two        wtab[k] = exp(-2 pi i k / 256), rounded (FP32) or split (double-float) once
+//   the others          the error flag of windows outside the object
+template <typename C>
+__global__ void __launch_bounds__(256) setup_kernel(const float* __restrict__ V, const float2* __restrict__ X, C* __restrict__ T,
+                                                    size_t n, double sigma, int nt, C* __restrict__ h1, int W, double dzlam,
+                                                    double dq, C* __restrict__ wtab, float2* __restrict__ wtab8,
+                                                    const int2* __restrict__ pos, int S, int Ny, int Nx, int* err) {
+  wait_for_predecessor();
+  const int tid = threadIdx.x;
+  int b = blockIdx.x;
+  if (b < nt) {
+    for (size_t i = b * (size_t)256 + tid; i < n; i += (size_t)nt * 256) {
+      if (X) {
+        T[i] = from_f2<C>(X[i]);
+      } else {
+        double sn, cs;
+        sincos(sigma * (double)V[i], &sn, &cs);
+        T[i] = from_d<C>(cs, sn);
+      }
+    }
+    return;
+  }
+  b -= nt;
+  if (b < W / 32) {
+    if (tid >= 32) return;
+    const int k = 32 * b + tid;
+    const double q = (double)(k < W / 2 ? k : k - W) * dq;
+    double t = dzlam * q * q;
+    t = t - 2.0 * floor(t * 0.5);
+    double sn, cs;
+    sincospi(t, &sn, &cs);
+    h1[k] = from_d<C>(cs / W, -sn / W);
+    return;
+  }
+  b -= W / 32;
+  if (b < 2) {
+    double sn, cs;
+    sincospi(2.0 * (double)tid / 256.0, &sn, &cs);
+    if (b == 0) wtab[tid] = from_d<C>(cs, -sn);
+    else wtab8[tid] = make_float2((float)cs, (float)-sn);
+    return;
+  }
+  const int i = (b - 2) * 256 + tid;
+  if (i < S && !window_ok(pos[i], Ny, Nx, W)) atomicMax(err, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -928,24 +935,20 @@ cudaError_t run_precise(int mode, const PosParams& p, int W, const PreciseIn& in
     if ((err = tcdft_prepare(W, 0, g.mat_f, st)) != cudaSuccess) return err;
     if ((err = tcdft_prepare(W, 1, g.mat_i, st)) != cudaSuccess) return err;
     n_launch += 2;
-  } else if (df) {
-    table64_kernel<dfc><<<elem_blocks((size_t)L * plane, in.sms), 256, 0, st>>>(in.X ? nullptr : in.V, in.X,
-                                                                                 (dfc*)g.T64, (size_t)L * plane,
-                                                                                 in.sigma);
-    h1_64_kernel<dfc><<<(W + 255) / 256, 256, 0, st>>>((dfc*)g.h1d, W, in.dzlam, in.dq);
-    wtab_kernel<dfc><<<1, 256, 0, st>>>((dfc*)g.wtab16);
-    wtab_kernel<float2><<<1, 256, 0, st>>>(g.wtab8);
-    n_launch += 4;
+    flag_windows_kernel<<<(S + 255) / 256, 256, 0, st>>>(p.pos, S, p.Ny, p.Nx, W, p.err);
+    ++n_launch;
   } else {
-    table64_kernel<double2><<<elem_blocks((size_t)L * plane, in.sms), 256, 0, st>>>(in.X ? nullptr : in.V, in.X,
-                                                                                     g.T64, (size_t)L * plane, in.sigma);
-    h1_64_kernel<double2><<<(W + 255) / 256, 256, 0, st>>>(g.h1d, W, in.dzlam, in.dq);
-    wtab_kernel<double2><<<1, 256, 0, st>>>((double2*)g.wtab16);
-    wtab_kernel<float2><<<1, 256, 0, st>>>(g.wtab8);
-    n_launch += 4;
+    const size_t n = (size_t)L * plane;
+    const int nt = elem_blocks(n, in.sms);
+    auto setup = [&](auto* T, auto* h1, auto* wtab) {
+      return launch_following(setup_kernel<std::remove_pointer_t<decltype(T)>>, dim3(nt + W / 32 + 2 + (S + 255) / 256), dim3(256),
+                              0, st, in.X ? nullptr : in.V, in.X, T, n, in.sigma, nt, h1, W, in.dzlam, in.dq, wtab, g.wtab8,
+                              p.pos, S, p.Ny, p.Nx, p.err);
+    };
+    err = df ? setup((dfc*)g.T64, (dfc*)g.h1d, (dfc*)g.wtab16) : setup((double2*)g.T64, (double2*)g.h1d, (double2*)g.wtab16);
+    if (err != cudaSuccess) return err;
+    ++n_launch;
   }
-  flag_windows_kernel<<<(S + 255) / 256, 256, 0, st>>>(p.pos, S, p.Ny, p.Nx, W, p.err);
-  ++n_launch;
 
   // 2-D transforms: unnormalised, forward or inverse
   auto keep_first = [&](cudaError_t e) {
@@ -1070,7 +1073,7 @@ cudaError_t run_precise(int mode, const PosParams& p, int W, const PreciseIn& in
       }
     }
     if (want_dprobe) {
-      dprobe_accumulate_kernel<<<(int)((WW + 255) / 256), 256, 0, st>>>(g.contrib, nb, (int)WW, g.dp64, b0 == 0);
+      dprobe_accumulate_kernel<<<(int)((WW + 63) / 64), 64, 0, st>>>(g.contrib, nb, (int)WW, g.dp64, b0 == 0);
       ++n_launch;
     }
   }
