@@ -615,7 +615,7 @@ def run_dft(args, rank, world, local_rank):
                      "kernel": "cgemm_kernel<false, true> (one DFT pass, tcgen05 kind::tf32, split operands)",
                      "kernel_ms": pass_ms,
                      "peak_source": "measured tcgen05 kind::tf32 pipe rate (bench.py --config peaks, N = 256)"},
-        "smem_fft_comparison": {"fused_kernel": "position_kernel<128, LAYER> on the c3 layer step",
+        "smem_fft_comparison": {"fused_kernel": "wave_kernel<128, LAYER> on the c3 layer step",
                                 "fused_kernel_ms": fused_ms, "fft_transforms_per_s": fft_rate,
                                 "tensor_dft_over_smem_fft": value / fft_rate},
         "e2e": {"value": e2e, "unit": DFT_UNIT, "h2d_bytes_per_step": S * W * W * 8, "d2h_bytes_per_step": S * W * W * 8},
@@ -1017,8 +1017,7 @@ def run_msp(args, rank, world, local_rank):
     fused_ms = prof["fused_ms"] / args.steps
     fused_launches_per_call = prof["fused_launches"] / args.steps
     achieved = fft_flops(S, L, W) / (fused_ms * 1e-3) / 1e12
-    kname = "position_kernel<128, LOSS_GRAD>" if W == 128 else ("position_cluster_kernel<LOSS_GRAD>" if W == 256
-                                                                 else f"position_kernel<{W}, LOSS_GRAD>")
+    kname = f"position_kernel<{W}, LOSS_GRAD>" if W == 64 else f"wave_kernel<{W}, LOSS_GRAD>"
     traffic = None
     if cfg is synth.C2:
         traffic = measured_traffic("position_kernel_loss_grad" + ("_l2_reduce" if args.overlap_add == "l2" else ""))

@@ -782,7 +782,7 @@ static msp_status prepare(const msp_geometry* g, const float* probe, const float
   const bool pot = g->param != MSP_PARAM_TRANSMISSION;   // transmission mode uses the caller's slices as given
   const size_t n = pot ? (size_t)g->n_slices * g->obj_ny * g->obj_nx : 0;
   const int blocks = 1 + W / 32 + (int)std::min<size_t>((n + 1023) / 1024, (size_t)c.dev.sms * 4);
-  MSP_CK(launch_following(prepare_kernel, dim3(blocks), dim3(1024), 0, c.st, (const float2*)probe, W,
+  MSP_CK(launch_following(prepare_kernel, dim3(blocks), dim3(1024), 0, c.st, 1, (const float2*)probe, W,
                           kZeroRuleTau * kZeroRuleTau, c.ws.scal + 5, c.ws.h1, g->dz_A * g->wavelength_A,
                           1.0 / ((double)W * g->pixel_A), c.ws.err, V, c.ws.T, n, (float)g->sigma));
   counted();
@@ -956,7 +956,7 @@ msp_status msp_loss_grad(const msp_geometry* g, const float* probe, const float*
   const int n_dprobe = dprobe ? (int)((WW + kDprobeVals - 1) / kDprobeVals) : 0;
   const int nblk = n_gather + n_dprobe + 1;
   MSP_CK(launch_following(p.cplx ? loss_grad_finish_kernel<true> : loss_grad_finish_kernel<false>, dim3(nblk), dim3(256), 0,
-                          c.st, c.ws.wgrad, (const int2*)pos, g->n_pos, W, g->n_slices, g->obj_ny, g->obj_nx, gx, gy, dV,
+                          c.st, 1, c.ws.wgrad, (const int2*)pos, g->n_pos, W, g->n_slices, g->obj_ny, g->obj_nx, gx, gy, dV,
                           n_gather, c.ws.dprobe_part, c.parts, (float2*)dprobe, n_dprobe, c.ws.loss_part,
                           g->n_pos * loss_slots(g), c.ws.scal, loss));
   counted();
@@ -1006,9 +1006,9 @@ msp_status msp_layer_step(const msp_geometry* g, const float* probe, float* V, c
   MSP_TRY(run_position(g, MODE_LAYER, p, c));
   float* tilemax = (float*)c.ws.red;
   if (l2_reduce)
-    MSP_CK(launch_following(tile_max_kernel, grid, dim3(256), 0, c.st, c.ws.map1, g->obj_ny, g->obj_nx, tilemax));
+    MSP_CK(launch_following(tile_max_kernel, grid, dim3(256), 0, c.st, 1, c.ws.map1, g->obj_ny, g->obj_nx, tilemax));
   else
-    MSP_CK(launch_following(p.cplx ? gather_kernel<true, true> : gather_kernel<false, true>, grid, dim3(256), 0, c.st,
+    MSP_CK(launch_following(p.cplx ? gather_kernel<true, true> : gather_kernel<false, true>, grid, dim3(256), 0, c.st, 1,
                             c.ws.wgrad, c.ws.willum, 1, (const int2*)pos, g->n_pos, W, g->obj_ny, g->obj_nx, c.ws.map0,
                             c.ws.map1, tilemax));
   counted();
@@ -1022,7 +1022,7 @@ msp_status msp_layer_step(const msp_geometry* g, const float* probe, float* V, c
   // V_l (or the complex o_l, as interleaved floats) -= mu * gradient map
   const size_t nupd = plane * (p.cplx ? 2 : 1);
   const int blocks = 1 + (int)std::min<size_t>((nupd + 255) / 256, (size_t)c.dev.sms);
-  MSP_CK(launch_following(layer_update_kernel, dim3(blocks), dim3(256), 0, c.st, V + (size_t)layer * nupd, c.ws.map0, nupd,
+  MSP_CK(launch_following(layer_update_kernel, dim3(blocks), dim3(256), 0, c.st, 1, V + (size_t)layer * nupd, c.ws.map0, nupd,
                           tilemax, nblk, c.ws.loss_part, g->n_pos * loss_slots(g), step, c_w2, p.cplx, c.ws.scal, mu_out,
                           loss_before));
   counted();
@@ -1058,7 +1058,7 @@ msp_status msp_probe_step(const msp_geometry* g, float* probe, const float* V, c
     p.want_dprobe = 1;
     MSP_TRY(run_position(g, MODE_PROBE, p, c));
     const int nb = (int)((WW + kDprobeVals - 1) / kDprobeVals);
-    MSP_CK(launch_following(probe_finish_kernel, dim3(nb + 1), dim3(256), 0, c.st, c.ws.dprobe_part, c.parts, (int)WW,
+    MSP_CK(launch_following(probe_finish_kernel, dim3(nb + 1), dim3(256), 0, c.st, 1, c.ws.dprobe_part, c.parts, (int)WW,
                             c.ws.dprobe_sum, normalize ? nullptr : (float2*)probe, mu, c.ws.loss_part,
                             g->n_pos * loss_slots(g), c.ws.scal, normalize ? nullptr : mu_out, loss_before));
     counted();

@@ -1,24 +1,23 @@
-// msp_fft.cuh -- 2-D FFT building blocks for sm_103a: line transforms by thread groups (W = 64, 256), small
-// transforms in registers (W = 128), and the residual of the far field.
+// msp_fft.cuh -- 2-D FFT building blocks for sm_103a: line transforms by groups of eight threads (W = 64),
+// small transforms in registers (W = 128, 256), and the residual of the far field.
 //
 // The Fourier operator F of the multislice model (Sec. 2.1 / 2.2) is the
-// unnormalised 2-D DFT of a W x W wave.  A W-point line transform is split
+// unnormalised 2-D DFT of a W x W wave.  A W-point line transform by a group is split
 // W = N1 * 8 (four-step Cooley-Tukey): eight threads share one line, thread j
 // holds the line elements j, j+8, j+16, ...  (N1 complex values in registers),
 //   step A: an N1-point DFT in registers over those elements,
 //   step B: twiddle by w_W^(j k1),
 //   exchange through a small shared buffer private to the group (warp-synchronous),
 //   step C: N1/8 eight-point DFTs in registers.
-// (W = 256 uses sixteen threads per line and sixteen-point DFTs in both steps.)
 // The output indices k1 + N1 k2 held by thread j are again exactly the set
 // {j + 8m}, so every line transform starts and ends with the same thread/index
 // ownership and consecutive passes need no re-distribution beyond the row <->
 // column transpose through shared memory.
 //
-// The inverse transform is conj(F(conj(x))) (unnormalised); negations fold into
+// There the inverse transform is conj(F(conj(x))) (unnormalised); negations fold into
 // the arithmetic, so one forward kernel of small DFTs serves both directions.
 //
-// Shared-memory layout of the wave: element (r, c) lives at r*W + (c ^ swz(r)),
+// Shared-memory layout of the W = 64 wave: element (r, c) lives at r*W + (c ^ swz(r)),
 // swz(r) = ((r & 1) << 3) | (r & 6).  With eight threads per line and four lines
 // per warp this makes every row and column access of the wave free of bank
 // conflicts for 8-byte elements.
@@ -134,15 +133,6 @@ __device__ __forceinline__ void dft(const float2* x, float2* X) {
 
 __device__ __forceinline__ int swz(int r) { return ((r & 1) << 3) | (r & 6); }
 
-// Twiddles w_W^(j k1) of thread j (of T per line), read from the shared table [k1 * T + j].
-template <int T = 8>
-struct SharedTwiddles {
-  const float2* __restrict__ t;
-  int j;
-  template <int K1>
-  __device__ __forceinline__ float2 get() const { return t[K1 * T + j]; }
-};
-
 // Twiddles of thread j held in registers: w^(j k) for k < 8, and w^(j k) = w^(8j) w^(j (k - 8))
 // for k >= 8 (one extra rounded product).  `t` is the shared table [k1 * T + j].
 template <int W, int T = 8>
@@ -170,17 +160,11 @@ __device__ __forceinline__ void twiddle_store(const float2* y, float2* xw, const
   }
 }
 
-// Line transform of a W-point line held by T threads (lane group, T = 8 or 16), in place
-// in `v`: on entry v[m] is line element j + T m, on exit v[m] is spectrum element j + T m.
-// W = N1 T (four-step): step A is an N1-point DFT in registers over x[T n1 + j], step B
-// the twiddles w_W^(j k1), then an exchange, then step C, N1/T T-point DFTs.
-// `xb` is the group's private exchange buffer of T * (N1 + 1) float2: thread j writes
-// its step-A results Y[j][k1] at xb[j (N1 + 1) + k1] and reads Y[n2][k1] at
-// xb[n2 (N1 + 1) + k1]; the odd stride N1 + 1 spreads both patterns over distinct banks
-// (and, for T = 8, consecutive groups' buffers start half a bank row apart), so the
-// exchange is conflict-free and its addresses are a per-thread base plus immediate offsets.
-// `tw.get<k1>()` = w_W^(j k1) (forward sign).  INV selects the unnormalised inverse.
-// Exchange layout with the step-A results transposed (eight threads per line): row k1 of
+// Line transform of a W-point line held by eight threads, in place in `v`: on entry v[m] is line element
+// j + 8 m, on exit v[m] is spectrum element j + 8 m.  W = 8 N1 (four-step): step A is an N1-point DFT in
+// registers over x[8 n1 + j], step B the twiddles w_W^(j k1), then an exchange, then step C, N1/8 eight-point
+// DFTs.  `tw.get<k1>()` = w_W^(j k1) (forward sign).  INV selects the unnormalised inverse.
+// Exchange layout with the step-A results transposed: row k1 of
 // the group's buffer holds Y[0..7][k1] at stride kXRow, so thread j writes Y[j][k1] at
 // xb[k1 kXRow + j] (64-bit stores) and reads its step-C operands Y[0..7][k1] for
 // k1 = j + 8 mc as four 128-bit loads per row.  With kXRow = 10 and group buffers
@@ -218,41 +202,6 @@ __device__ __forceinline__ void line_fft_t(float2 (&v)[W / 8], const Tw& tw, flo
     dft<8, 1>(b[mc], X);
 #pragma unroll
     for (int k2 = 0; k2 < 8; ++k2) v[mc + NC * k2] = INV ? cconj(X[k2]) : X[k2];
-  }
-}
-
-template <int W, bool INV, typename Tw, int T = 8>
-__device__ __forceinline__ void line_fft(float2 (&v)[W / T], const Tw& tw, float2* xb, int j) {
-  constexpr int N1 = W / T;
-  constexpr int NC = N1 / T;
-  constexpr int XS = N1 + 1;
-  static_assert(N1 % T == 0, "W / T must be a multiple of T");
-  float2 y[N1];
-  if constexpr (INV) {
-#pragma unroll
-    for (int m = 0; m < N1; ++m) v[m] = cconj(v[m]);
-  }
-  // step A: DFT over n1 of x[T n1 + j]
-  dft<N1, 1>(v, y);
-  // step B: twiddles, then exchange Y[n2 = j][k1]
-  float2* xw = xb + j * XS;
-  twiddle_store<0, N1>(y, xw, tw);
-  __syncwarp();
-  float2 b[NC][T];
-  const float2* xr = xb + j;
-#pragma unroll
-  for (int mc = 0; mc < NC; ++mc) {
-#pragma unroll
-    for (int n2 = 0; n2 < T; ++n2) b[mc][n2] = xr[n2 * XS + T * mc];
-  }
-  __syncwarp();   // the buffer is reused by this group's next transform
-  // step C: T-point DFTs over n2; X[k1 + N1 k2] with k1 = j + T mc is v[mc + NC k2]
-#pragma unroll
-  for (int mc = 0; mc < NC; ++mc) {
-    float2 X[T];
-    dft<T, 1>(b[mc], X);
-#pragma unroll
-    for (int k2 = 0; k2 < T; ++k2) v[mc + NC * k2] = INV ? cconj(X[k2]) : X[k2];
   }
 }
 
@@ -339,6 +288,8 @@ MSP_PACKED_OP(add2, "add.rn.f32x2")
 MSP_PACKED_OP(sub2, "sub.rn.f32x2")
 MSP_PACKED_OP(mul2, "mul.rn.f32x2")
 #undef MSP_PACKED_OP
+
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
 // Two complex values side by side, (re0, re1) and (im0, im1).
 struct C2 {

@@ -139,7 +139,6 @@ struct alignas(16) dfc {
   __device__ __forceinline__ dff re() const { return {h.x, l.x}; }
   __device__ __forceinline__ dff im() const { return {h.y, l.y}; }
 };
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
 __device__ __forceinline__ dfc fast_two_sum(float2 a, float2 b) {
   const float2 s = add2(a, b);
@@ -942,7 +941,7 @@ cudaError_t run_precise(int mode, const PosParams& p, int W, const PreciseIn& in
     const int nt = elem_blocks(n, in.sms);
     auto setup = [&](auto* T, auto* h1, auto* wtab) {
       return launch_following(setup_kernel<std::remove_pointer_t<decltype(T)>>, dim3(nt + W / 32 + 2 + (S + 255) / 256), dim3(256),
-                              0, st, in.X ? nullptr : in.V, in.X, T, n, in.sigma, nt, h1, W, in.dzlam, in.dq, wtab, g.wtab8,
+                              0, st, 1, in.X ? nullptr : in.V, in.X, T, n, in.sigma, nt, h1, W, in.dzlam, in.dq, wtab, g.wtab8,
                               p.pos, S, p.Ny, p.Nx, p.err);
     };
     err = df ? setup((dfc*)g.T64, (dfc*)g.h1d, (dfc*)g.wtab16) : setup((double2*)g.T64, (double2*)g.h1d, (double2*)g.wtab16);
