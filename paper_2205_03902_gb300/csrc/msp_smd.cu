@@ -39,6 +39,7 @@
 #include "msp.h"
 #include "msp_smd.h"
 #include "msp_cgemm.cuh"
+#include "msp_kernels.cuh"
 
 namespace msp {
 
@@ -278,6 +279,7 @@ __global__ void __launch_bounds__(threads_of(N)) farfield_kernel(float2* BC, int
   const int t = threadIdx.x, r0 = 2 * (t / fac1(N)), c0 = t % fac1(N);
   fill_twiddles<N>(Wt);
   Twiddles<N> tw(Wt, c0);
+  wait_for_predecessor();
   const float thr2 = (float)scal[S_THR2];
   double obj = 0.0;
   for (int s = blockIdx.x; s < S; s += gridDim.x) {
@@ -412,6 +414,7 @@ __global__ void __launch_bounds__(threads_of(N)) grad_kernel(const float2* __res
   const int t = threadIdx.x, r0 = 2 * (t / fac1(N)), c0 = t % fac1(N);
   fill_twiddles<N>(Wt);
   Twiddles<N> tw(Wt, c0);
+  wait_for_predecessor();
   {
     const int chunk = (n2 + gridDim.x - 1) / gridDim.x;
     const int k0 = blockIdx.x * chunk, k1 = min(n2, k0 + chunk);
@@ -513,6 +516,7 @@ __global__ void __launch_bounds__(threads_of(N)) transfer_kernel(float2* A, cons
   const int t = threadIdx.x, r0 = 2 * (t / fac1(N)), c0 = t % fac1(N);
   fill_twiddles<N>(Wt);
   Twiddles<N> tw(Wt, c0);
+  wait_for_predecessor();
   double dot = 0.0, nrm = 0.0;
   for (int col = blockIdx.x; col < n2; col += gridDim.x) {
     float2 v[2][fac2(N)];
@@ -544,43 +548,71 @@ __global__ void __launch_bounds__(threads_of(N)) transfer_kernel(float2* A, cons
   }
 }
 
-// Matrix-step set-up (one CTA): max_k |(F p)_k|^2, the sum of I from its partials, the
-// squared zero-rule threshold and mu.
+// Matrix-step set-up: block 0 takes max_k |(F p)_k|^2, the others the sum of I over fixed chunks; the block that
+// is done last (a ticket, zeroed with the error word) adds the chunks in their order and forms the squared
+// zero-rule threshold and mu.  Both parts are short chains on few SMs (at N = 40 and 1600 positions 13.4 us for the
+// one image, 7.5 us for the 10 MB of I, as two launches one after the other), so they run side by side: 14.3 us.
+// A thread adds eight counts at a time in FP32 and these sums in FP64.
 template <int N>
 __global__ void __launch_bounds__(threads_of(N)) setup_kernel(const float2* __restrict__ probe,
-                                                              const double* __restrict__ sum_part, int n_part,
-                                                              double count, double step, double* scal,
-                                                              double* mu_out) {
+                                                              const float* __restrict__ I, size_t count, double step,
+                                                              double* sum_part, int* ticket, double* scal) {
   extern __shared__ float4 smem4[];
   float2* X = reinterpret_cast<float2*>(smem4);
   float2* Y = X + N * ld_of(N);
   float2* Wt = Y + N * ld_of(N);
   double* red = reinterpret_cast<double*>(Wt + tw_elems(N));
-  const int t = threadIdx.x, r0 = 2 * (t / fac1(N)), c0 = t % fac1(N);
-  fill_twiddles<N>(Wt);
-  Twiddles<N> tw(Wt, c0);
-  float2 v[2][fac2(N)];
+  __shared__ int last;
+  const int t = threadIdx.x, n_part = (int)gridDim.x - 1;
+  if (blockIdx.x == 0) {
+    const int r0 = 2 * (t / fac1(N)), c0 = t % fac1(N);
+    fill_twiddles<N>(Wt);
+    Twiddles<N> tw(Wt, c0);
+    wait_for_predecessor();
+    float2 v[2][fac2(N)];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < fac2(N); ++j) v[i][j] = probe[owned(N, r0, c0, i, j)];
-  dft2<N>(v, X, Y, tw, false, r0, c0);
-  double mx = 0.0;
+      for (int j = 0; j < fac2(N); ++j) v[i][j] = probe[owned(N, r0, c0, i, j)];
+    dft2<N>(v, X, Y, tw, false, r0, c0);
+    double mx = 0.0;
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < fac2(N); ++j) mx = fmax(mx, (double)v[i][j].x * v[i][j].x + (double)v[i][j].y * v[i][j].y);
-  const double m = block_sum<true>(mx, red);
+      for (int j = 0; j < fac2(N); ++j) mx = fmax(mx, (double)v[i][j].x * v[i][j].x + (double)v[i][j].y * v[i][j].y);
+    const double m = block_sum<true>(mx, red);
+    if (t == 0) scal[S_SPEC] = m;
+  } else {
+    wait_for_predecessor();
+    const size_t chunk = (count + n_part - 1) / n_part;
+    const size_t b0 = (blockIdx.x - 1) * chunk, b1 = min(count, b0 + chunk), nt = blockDim.x;
+    double a = 0.0;
+    size_t i = b0 + t;
+    for (; i + 7 * nt < b1; i += 8 * nt) {
+      float f[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) f[u] = __ldg(&I[i + u * nt]);
+      a += (double)(((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])));
+    }
+    for (; i < b1; i += nt) a += (double)__ldg(&I[i]);
+    const double tot = block_sum(a, red);
+    if (t == 0) sum_part[blockIdx.x - 1] = tot;
+  }
+  if (t == 0) {
+    __threadfence();
+    last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
   double a = 0.0;
-  for (int i = t; i < n_part; i += blockDim.x) a += sum_part[i];
+  for (int i = t; i < n_part; i += blockDim.x) a += __ldcg(&sum_part[i]);
   const double s = block_sum(a, red);
   if (t == 0) {
-    scal[S_SPEC] = m;
+    const double m = __ldcg(&scal[S_SPEC]);
     scal[S_SUMI] = s;
-    scal[S_THR2] = kZeroTau * kZeroTau * s / count;
-    const double mu = step > 0.0 ? step : (m > 0.0 ? 1.0 / ((double)(N * N) * m) : 0.0);
-    scal[S_MU] = mu;
-    if (mu_out) mu_out[0] = mu;
+    scal[S_THR2] = kZeroTau * kZeroTau * s / (double)count;
+    scal[S_MU] = step > 0.0 ? step : (m > 0.0 ? 1.0 / ((double)(N * N) * m) : 0.0);
   }
 }
 
@@ -595,6 +627,7 @@ constexpr int kProbeShifts = 128;   // shifts per block at most: S <= 128 gridDi
 __global__ void probe_matrix_kernel(const float2* __restrict__ probe, const int2* __restrict__ shifts, int N, int S,
                                     float2* __restrict__ P) {
   __shared__ int2 sh[kProbeShifts];
+  wait_for_predecessor();
   const int mine = (S - (int)blockIdx.y + (int)gridDim.y - 1) / (int)gridDim.y;   // shifts of this block
   for (int i = threadIdx.x; i < mine; i += blockDim.x) {
     const int2 v = shifts[blockIdx.y + i * gridDim.y];
@@ -620,36 +653,33 @@ __global__ void probe_matrix_kernel(const float2* __restrict__ probe, const int2
 // The propagator h[ky][kx] = exp(-i pi dz lambda (qy^2 + qx^2)) / N^2 = h1(ky) h1(kx) / N^2 and
 // its real-space kernel gk = G e_0, gk[y][x] = g1(y) g1(x), g1(y) = (1/N) sum_k h1(k)
 // exp(2 pi i k y / N), are outer products of one-dimensional factors: this kernel forms g1[y]
-// and h1[y] in double (one block of one warp per y, spreading the FP64 work over N SMs: lanes
-// take k = lane, lane + 32, then a butterfly sum), `kernel_column_kernel` the products.
-__global__ void __launch_bounds__(32) kernel_row_kernel(double2* __restrict__ g1, double2* __restrict__ h1, int N,
+// and h1[y] in double, `kernel_column_kernel` the products.  One block per y spreads the FP64 work over N
+// SMs, and a thread has at most one FP64 sincospi (one warp with three in a row: 10 us; so 5.5 us): warps 0 and 1 take
+// the terms k of the sum, thread 64 h1[y].
+__global__ void __launch_bounds__(96) kernel_row_kernel(double2* __restrict__ g1, double2* __restrict__ h1, int N,
                                                         double dzlam, double dq) {
-  const int y = blockIdx.x, lane = threadIdx.x;
-  double re = 0.0, im = 0.0;
-  for (int k = lane; k < N; k += 32) {
-    const double q = (k < N / 2 ? k : k - N) * dq;
-    double s, c;
-    sincospi(-dzlam * q * q + 2.0 * (double)((k * y) % N) / N, &s, &c);
-    re += c;
-    im += s;
-  }
+  __shared__ double2 half;
+  const int y = blockIdx.x, t = threadIdx.x;
+  const int k = t < 64 ? t : y;
+  const double q = (k < N / 2 ? k : k - N) * dq;
+  double s = 0.0, c = 0.0;
+  if (t < N || t == 64) sincospi(-dzlam * q * q + (t < 64 ? 2.0 * (double)((k * y) % N) / N : 0.0), &s, &c);
+  wait_for_predecessor();
+  if (t == 64) h1[y] = make_double2(c, s);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
-    re += __shfl_xor_sync(0xffffffffu, re, off);
-    im += __shfl_xor_sync(0xffffffffu, im, off);
+    c += __shfl_xor_sync(0xffffffffu, c, off);
+    s += __shfl_xor_sync(0xffffffffu, s, off);
   }
-  if (lane == 0) {
-    g1[y] = make_double2(re / N, im / N);
-    const double q = (y < N / 2 ? y : y - N) * dq;
-    double s, c;
-    sincospi(-dzlam * q * q, &s, &c);
-    h1[y] = make_double2(c, s);
-  }
+  if (t == 32) half = make_double2(c, s);
+  __syncthreads();
+  if (t == 0) g1[y] = make_double2((c + half.x) / N, (s + half.y) / N);
 }
 
 // gk[y][x] = g1(y) g1(x) and h[ky][kx] = h1(ky) h1(kx) / N^2, in double, each rounded once.
 __global__ void kernel_column_kernel(float2* __restrict__ gk, float2* __restrict__ h, const double2* __restrict__ g1,
                                      const double2* __restrict__ h1, int N) {
+  wait_for_predecessor();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= N * N) return;
   const double2 a = g1[e / N], b = g1[e % N];
@@ -659,23 +689,11 @@ __global__ void kernel_column_kernel(float2* __restrict__ gk, float2* __restrict
   h[e] = make_float2((float)((u.x * v.x - u.y * v.y) * inv), (float)((u.x * v.y + u.y * v.x) * inv));
 }
 
-// Block partial sums of a float array over fixed chunks: FP32 within a thread (a few dozen
-// terms), FP64 across the block.  Only the zero-rule threshold uses the total.
-__global__ void __launch_bounds__(256) sum_part_kernel(const float* __restrict__ x, size_t n, double* __restrict__ part) {
-  __shared__ double sh[257];
-  const size_t chunk = (n + gridDim.x - 1) / gridDim.x;
-  const size_t b0 = blockIdx.x * chunk, b1 = min(n, b0 + chunk);
-  float a = 0.f;
-#pragma unroll 8
-  for (size_t i = b0 + threadIdx.x; i < b1; i += 256) a += __ldg(&x[i]);
-  const double tot = block_sum((double)a, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
 // out = sum of part[0..n) in a fixed order (one block of 256), written to scal[slot] and copy.
 __global__ void __launch_bounds__(256) finish_sum_kernel(const double* __restrict__ part, int n, double* scal,
                                                          int slot, double* copy) {
   __shared__ double sh[257];
+  wait_for_predecessor();
   double a = 0.0;
   for (int i = threadIdx.x; i < n; i += 256) a += part[i];
   const double s = block_sum(a, sh);
@@ -688,6 +706,7 @@ __global__ void __launch_bounds__(256) finish_sum_kernel(const double* __restric
 // A += -mu * sum_z part_z (the rank-S update of the matrix step), float4 over element pairs.
 __global__ void combine_kernel(float2* __restrict__ A, const float2* __restrict__ part, int splits, size_t stride,
                                size_t n_pairs, const double* __restrict__ scal) {
+  wait_for_predecessor();
   const float a = (float)(-scal[S_MU]);
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n_pairs; e += (size_t)gridDim.x * blockDim.x) {
     float4 s = reinterpret_cast<const float4*>(part)[e];
@@ -706,52 +725,58 @@ __global__ void combine_kernel(float2* __restrict__ A, const float2* __restrict_
 
 // The proximal step (Eq. Prox_Min) before its normalisation.  Element e = l n2 + k of the
 // slices (a block: 32 elements of one slice; n2 is a multiple of 32):
-//   g_l[k]: slice 0 from g0, slices 1..M-1 summed in FP64 over the CTAs' partials in a fixed
-//           order (8 groups of CTAs, cta mod 8, then the groups in order);
+//   g_l[k]: slice 0 from g0, slices 1..M-1 summed over the CTAs' partials in a fixed order (32
+//           groups of CTAs, cta mod 32, then the groups in order), in compensated FP32: the FP64
+//           pipe converts and adds about one element per cycle and SM, and the 2 M of them at
+//           N = 40 made this kernel 23 us (26 us with the chain a quarter as long); 9.5 us so;
 //   x = o_l[k] - mu_l lambda g_l[k] in FP64, mu_l = 1 / (lambda prod_{m != l} max|o_m|)^2,
 //       written over o_l[k];
 //   normpart[block] = sum of |x|^2 over the block's 32 elements (fixed order).
-// max|o_m| comes from the CTAs' maxima (every block reduces them alike).  Block 0 also sums the
-// decomposition objective into scal[S_DOBJ] (and obj_out).
-__global__ void __launch_bounds__(256) grad_step_kernel(float2* __restrict__ o, const float2* __restrict__ g0,
+// max|o_m| comes from the CTAs' maxima (warp m of every block reduces them alike).  Block 0 also sums
+// the decomposition objective into scal[S_DOBJ] (and obj_out).
+constexpr int kGroups = 32;
+__global__ void __launch_bounds__(32 * kGroups) grad_step_kernel(float2* __restrict__ o, const float2* __restrict__ g0,
                                                         const float2* __restrict__ gpart,
                                                         const float* __restrict__ maxpart, int n_cta, int M, int n2,
                                                         const double* __restrict__ lam_p,
                                                         const double* __restrict__ obj_part,
                                                         double* __restrict__ normpart, double* scal,
                                                         double* obj_out) {
-  __shared__ double2 sh[8][32];
-  __shared__ double red[257];
+  __shared__ float4 sh[kGroups][32];   // (re.s, re.e, im.s, im.e)
+  __shared__ double red[32 * kGroups + 1];
   __shared__ double maxo[kMaxSlices];
   const int t = threadIdx.x, lane = t & 31, grp = t >> 5;
-  for (int m = 0; m < M; ++m) {
+  wait_for_predecessor();
+  if (grp < M) {
     float a = 0.f;
-    for (int c = t; c < n_cta; c += 256) a = fmaxf(a, maxpart[c * M + m]);
-    const double mx = block_sum<true>((double)a, red);
-    if (t == 0) maxo[m] = sqrt(mx);
+    for (int c = lane; c < n_cta; c += 32) a = fmaxf(a, maxpart[c * M + grp]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, off));
+    if (lane == 0) maxo[grp] = sqrt((double)a);
   }
   const int l = (blockIdx.x * 32) / n2, k = blockIdx.x * 32 - l * n2 + lane;
   const size_t na = (size_t)(M - 1) * n2;
-  double re = 0.0, im = 0.0;
+  Compensated re, im;
   if (l > 0)
-#pragma unroll 4
-    for (int c = grp; c < n_cta; c += 8) {
+#pragma unroll 5
+    for (int c = grp; c < n_cta; c += kGroups) {
       const float2 v = gpart[(size_t)c * na + (size_t)(l - 1) * n2 + k];
-      re += v.x;
-      im += v.y;
+      re.add(v.x);
+      im.add(v.y);
     }
-  sh[grp][lane] = make_double2(re, im);
+  sh[grp][lane] = make_float4(re.s, re.e, im.s, im.e);
   __syncthreads();
   if (grp == 0) {
     double2 g;
     if (l == 0) {
       g = make_double2(g0[k].x, g0[k].y);
     } else {
-      g = sh[0][lane];
-      for (int q = 1; q < 8; ++q) {
-        g.x += sh[q][lane].x;
-        g.y += sh[q][lane].y;
+      for (int q = 1; q < kGroups; ++q) {
+        const float4 v = sh[q][lane];
+        re.add(Compensated{v.x, v.y});
+        im.add(Compensated{v.z, v.w});
       }
+      g = make_double2(re.wide(), im.wide());
     }
     const double lam = lam_p[0];
     double bound = fabs(lam);
@@ -768,7 +793,7 @@ __global__ void __launch_bounds__(256) grad_step_kernel(float2* __restrict__ o, 
   }
   if (blockIdx.x == 0) {
     double a = 0.0;
-    for (int i = t; i < n_cta; i += 256) a += obj_part[i];
+    for (int i = t; i < n_cta; i += 32 * kGroups) a += obj_part[i];
     const double tot = block_sum(a, red);
     if (t == 0) {
       scal[S_DOBJ] = tot;
@@ -782,6 +807,7 @@ __global__ void __launch_bounds__(256) grad_step_kernel(float2* __restrict__ o, 
 __global__ void __launch_bounds__(256) prox_kernel(float2* __restrict__ o, const double* __restrict__ normpart,
                                                    int n2) {
   __shared__ double red[257];
+  wait_for_predecessor();
   const int l = blockIdx.y, nb = n2 / 32;
   double a = 0.0;
   for (int i = threadIdx.x; i < nb; i += 256) a += normpart[l * nb + i];
@@ -797,6 +823,7 @@ __global__ void __launch_bounds__(256) prox_kernel(float2* __restrict__ o, const
 __global__ void __launch_bounds__(256) lambda_kernel(const double* __restrict__ dot_part,
                                                      const double* __restrict__ nrm_part, int n, double* lam) {
   __shared__ double sh[257];
+  wait_for_predecessor();
   double d = 0.0, q = 0.0;
   for (int i = threadIdx.x; i < n; i += 256) {
     d += dot_part[i];
@@ -808,6 +835,7 @@ __global__ void __launch_bounds__(256) lambda_kernel(const double* __restrict__ 
 }
 
 __global__ void scale_kernel(float4* __restrict__ A, size_t n4, const double* __restrict__ lam) {
+  wait_for_predecessor();
   const float s = (float)lam[0];
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n4; e += (size_t)gridDim.x * blockDim.x) {
     float4 v = A[e];
@@ -1079,10 +1107,11 @@ static msp_status begin(const msp_smd_geometry* g, void* ws, size_t ws_bytes, vo
 
 static msp_status launch_propagator(const msp_smd_geometry* g, Call& c) {
   const int N = g->n;
-  kernel_row_kernel<<<N, 32, 0, c.st>>>(c.w.g1, c.w.g1 + 64, N, g->dz_A * g->wavelength_A,
-                                        1.0 / ((double)N * g->pixel_A));
+  SMD_CK(launch_following(kernel_row_kernel, dim3(N), dim3(96), 0, c.st, 1, c.w.g1, c.w.g1 + 64, N,
+                          g->dz_A * g->wavelength_A, 1.0 / ((double)N * g->pixel_A)));
   SMD_LAUNCHED(1);
-  kernel_column_kernel<<<(N * N + 255) / 256, 256, 0, c.st>>>(c.w.gk, c.w.h, c.w.g1, c.w.g1 + 64, N);
+  SMD_CK(launch_following(kernel_column_kernel, dim3((N * N + 255) / 256), dim3(256), 0, c.st, 1, c.w.gk, c.w.h, c.w.g1,
+                          c.w.g1 + 64, N));
   SMD_LAUNCHED(1);
   return MSP_OK;
 }
@@ -1092,11 +1121,11 @@ static msp_status launch_transfer(const msp_smd_geometry* g, Call& c, float2* A,
                                   bool have_ahat) {
   const size_t sm = Kernels<N>::smem_plain();
   if (have_ahat)
-    transfer_kernel<N, true><<<c.w.grid_plain, threads_of(N), sm, c.st>>>(A, o, c.w.gk, c.w.h, g->n_slices, scale,
-                                                                          c.w.part, c.w.part2);
+    SMD_CK(launch_following(transfer_kernel<N, true>, dim3(c.w.grid_plain), dim3(threads_of(N)), sm, c.st, 1, A, o,
+                            c.w.gk, c.w.h, g->n_slices, scale, c.w.part, c.w.part2));
   else
-    transfer_kernel<N, false><<<c.w.grid_plain, threads_of(N), sm, c.st>>>(A, o, c.w.gk, c.w.h, g->n_slices, scale,
-                                                                           nullptr, nullptr);
+    SMD_CK(launch_following(transfer_kernel<N, false>, dim3(c.w.grid_plain), dim3(threads_of(N)), sm, c.st, 1, A, o,
+                            c.w.gk, c.w.h, g->n_slices, scale, nullptr, nullptr));
   SMD_LAUNCHED(1);
   return MSP_OK;
 }
@@ -1106,17 +1135,15 @@ static msp_status matrix_step_n(const msp_smd_geometry* g, Call& c, float2* A, c
                                 const int2* shifts, const float* I, double step, double* obj_out) {
   const size_t n2 = (size_t)N * N, S = g->n_pos;
   const Layout& w = c.w;
-  SMD_CK(cudaMemsetAsync(w.err, 0, sizeof(int), c.st));   // the call's own error word
+  SMD_CK(cudaMemsetAsync(w.err, 0, 2 * sizeof(int), c.st));   // the call's own error word and the set-up's ticket
   // every block takes at most kProbeShifts shifts: gridDim.y >= S / kProbeShifts
   const unsigned gy = (unsigned)std::min<size_t>(S, std::max<size_t>(128, (S + kProbeShifts - 1) / kProbeShifts));
-  probe_matrix_kernel<<<dim3((unsigned)((n2 + 255) / 256), gy), 256, 0, c.st>>>(
-      probe, shifts, N, (int)S, w.P);
+  SMD_CK(launch_following(probe_matrix_kernel, dim3((unsigned)((n2 + 255) / 256), gy), dim3(256), 0, c.st, 1, probe,
+                          shifts, N, (int)S, w.P));
   SMD_LAUNCHED(1);
   const int nsum = std::min(kPartSlots, 4 * c.dev.sms);
-  sum_part_kernel<<<nsum, 256, 0, c.st>>>(I, n2 * S, w.part2);
-  SMD_LAUNCHED(1);
-  setup_kernel<N><<<1, threads_of(N), Kernels<N>::smem_plain(), c.st>>>(probe, w.part2, nsum, (double)(n2 * S), step,
-                                                                        w.scal, nullptr);
+  SMD_CK(launch_following(setup_kernel<N>, dim3(1 + nsum), dim3(threads_of(N)), Kernels<N>::smem_plain(), c.st, 1, probe, I,
+                          n2 * S, step, w.part2, w.err + 1, w.scal));
   SMD_LAUNCHED(1);
   // A P: M = N^2, N = S, K = N^2
   dim3 g1((unsigned)((n2 + gemm::TM - 1) / gemm::TM), (unsigned)((S + gemm::TN - 1) / gemm::TN), (unsigned)w.s1.splits);
@@ -1125,10 +1152,10 @@ static msp_status matrix_step_n(const msp_smd_geometry* g, Call& c, float2* A, c
                                                                          w.P, n2, w.BC, n2, n2 * S, w.err, tc_wait_limit());
     return cudaGetLastError();
   }));
-  farfield_kernel<N><<<w.grid_ff, threads_of(N), Kernels<N>::smem_plain(), c.st>>>(w.BC, w.s1.splits, n2 * S, I,
-                                                                                   (int)S, w.scal, w.part);
+  SMD_CK(launch_following(farfield_kernel<N>, dim3(w.grid_ff), dim3(threads_of(N)), Kernels<N>::smem_plain(), c.st, 1,
+                          w.BC, w.s1.splits, n2 * S, I, (int)S, w.scal, w.part));
   SMD_LAUNCHED(1);
-  finish_sum_kernel<<<1, 256, 0, c.st>>>(w.part, w.grid_ff, w.scal, S_OBJ, obj_out);
+  SMD_CK(launch_following(finish_sum_kernel, dim3(1), dim3(256), 0, c.st, 1, w.part, w.grid_ff, w.scal, S_OBJ, obj_out));
   SMD_LAUNCHED(1);
   // C P^H: M = N^2, N = N^2, K = S
   dim3 g2((unsigned)((n2 + gemm::TM - 1) / gemm::TM), (unsigned)((n2 + gemm::TN - 1) / gemm::TN), (unsigned)w.s2.splits);
@@ -1138,8 +1165,8 @@ static msp_status matrix_step_n(const msp_smd_geometry* g, Call& c, float2* A, c
     return cudaGetLastError();
   }));
   const size_t pairs = n2 * n2 / 2;
-  combine_kernel<<<(int)std::min<size_t>((pairs + 255) / 256, (size_t)c.dev.sms * 16), 256, 0, c.st>>>(
-      A, w.U, w.s2.splits, n2 * n2, pairs, w.scal);
+  SMD_CK(launch_following(combine_kernel, dim3((unsigned)std::min<size_t>((pairs + 255) / 256, (size_t)c.dev.sms * 16)),
+                          dim3(256), 0, c.st, 1, A, w.U, w.s2.splits, n2 * n2, pairs, w.scal));
   SMD_LAUNCHED(1);
   return MSP_OK;
 }
@@ -1148,9 +1175,8 @@ template <int N, int M>
 static cudaError_t launch_grad_m(Call& c, const float2* A, const float2* o, const double* lam) {
   if constexpr (M <= max_slices(N)) {
     const Layout& w = c.w;
-    grad_kernel<N, M><<<w.grid_grad, threads_of(N), Kernels<N>::smem_grad(M), c.st>>>(A, o, w.gk, w.h, lam, w.g0,
-                                                                                      w.gpart, w.part, w.maxpart);
-    return cudaGetLastError();
+    return launch_following(grad_kernel<N, M>, dim3(w.grid_grad), dim3(threads_of(N)), Kernels<N>::smem_grad(M), c.st, 1,
+                            A, o, w.gk, w.h, lam, w.g0, w.gpart, w.part, w.maxpart);
   }
   return cudaErrorInvalidValue;
 }
@@ -1177,16 +1203,18 @@ static msp_status decompose_n(const msp_smd_geometry* g, Call& c, float2* A, flo
   SMD_TRY(launch_propagator(g, c));
   SMD_TRY(launch_grad<N>(M, c, A, o, lam));
   SMD_LAUNCHED(1);
-  grad_step_kernel<<<(int)(M * n2 / 32), 256, 0, c.st>>>(o, w.g0, w.gpart, w.maxpart, w.grid_grad, M, (int)n2, lam,
-                                                        w.part, w.normpart, w.scal, obj_out);
+  SMD_CK(launch_following(grad_step_kernel, dim3((unsigned)(M * n2 / 32)), dim3(32 * kGroups), 0, c.st, 1, o, w.g0, w.gpart,
+                          w.maxpart, w.grid_grad, M, (int)n2, lam, w.part, w.normpart, w.scal, obj_out));
   SMD_LAUNCHED(1);
-  prox_kernel<<<dim3((unsigned)((n2 + 255) / 256), (unsigned)M), 256, 0, c.st>>>(o, w.normpart, (int)n2);
+  SMD_CK(launch_following(prox_kernel, dim3((unsigned)((n2 + 255) / 256), (unsigned)M), dim3(256), 0, c.st, 1, o,
+                          w.normpart, (int)n2));
   SMD_LAUNCHED(1);
   SMD_TRY(launch_transfer<N>(g, c, A, o, 1.f, true));
-  lambda_kernel<<<1, 256, 0, c.st>>>(w.part, w.part2, w.grid_plain, lam);
+  SMD_CK(launch_following(lambda_kernel, dim3(1), dim3(256), 0, c.st, 1, w.part, w.part2, w.grid_plain, lam));
   SMD_LAUNCHED(1);
   const size_t n4 = n2 * n2 / 2;
-  scale_kernel<<<(int)std::min<size_t>((n4 + 255) / 256, (size_t)c.dev.sms * 16), 256, 0, c.st>>>((float4*)A, n4, lam);
+  SMD_CK(launch_following(scale_kernel, dim3((unsigned)std::min<size_t>((n4 + 255) / 256, (size_t)c.dev.sms * 16)),
+                          dim3(256), 0, c.st, 1, (float4*)A, n4, lam));
   SMD_LAUNCHED(1);
   return MSP_OK;
 }
