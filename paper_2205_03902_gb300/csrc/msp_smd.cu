@@ -777,6 +777,14 @@ __global__ void __launch_bounds__(32 * kGroups) grad_step_kernel(float2* __restr
         im.add(Compensated{v.z, v.w});
       }
       g = make_double2(re.wide(), im.wide());
+      if (!isfinite(g.x) || !isfinite(g.y)) {   // a partial, or only its FP32 sum: FP64 tells
+        g = make_double2(0.0, 0.0);
+        for (int c = 0; c < n_cta; ++c) {
+          const float2 v = gpart[(size_t)c * na + (size_t)(l - 1) * n2 + k];
+          g.x += v.x;
+          g.y += v.y;
+        }
+      }
     }
     const double lam = lam_p[0];
     double bound = fabs(lam);

@@ -1,5 +1,5 @@
-"""The W = 128 kernel where its schedule changes (slices in tensor memory, windows fetched ahead, skipped
-positions, CTAs with one, two and three positions) and the far-field residual on operands that are not finite.
+"""The W = 128 and W = 256 kernels where their schedule changes (slices in tensor memory, windows fetched ahead, skipped
+positions, CTAs and clusters with one, two and three positions) and the far-field residual on operands that are not finite.
 
 Every position uses one of a few windows, so the oracle needs one evaluation per window.  The state is far from
 the data (kappa ~ 1), where the FP32 forward's rounding is not amplified: the bar is the 1e-5 of
@@ -45,7 +45,7 @@ class Problem:
         if cplx:
             t = (1 + 0.1 * rng.standard_normal((L, ny, nx))) * np.exp(1j * self.gd["sigma"] * self.V)
             self.T = t.astype(np.complex64).astype(np.complex128)
-        p = synth.probe(synth.C2 if win == 128 else synth.C1, norm2=50.0)[:win, :win]
+        p = synth.probe({64: synth.C1, 128: synth.C2, 256: synth.C4}[win], norm2=50.0)[:win, :win]
         self.probe = p.astype(np.complex64).astype(np.complex128)
         self.windows = np.asarray(windows, dtype=np.int32)
         self.I = rng.poisson(3.0, size=(len(windows), win, win)).astype(np.float64)
@@ -100,7 +100,51 @@ def test_positions_of_a_cta_skipped_first_last_and_in_a_row(msp, L):
         assert not out[b].any()
 
 
-@pytest.mark.parametrize("win", [64, 128])
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("L", [1, 2, 5])
+def test_slices_of_a_cluster(msp, L, cplx):
+    q = Problem(256, L, [(0, 0), (5, 3), (1, 11)], (261, 267), cplx)
+    _, (loss, dV, dp), good = q.run(msp, np.arange(5) % 3)
+    el, eV, ep = q.expect(good)
+    assert abs(float(loss) / el - 1) < TOL and rel(dV.cpu(), eV) < TOL and rel(dp.cpu(), ep) < TOL
+
+
+def test_positions_of_a_cluster_skipped_first_last_and_in_a_row(msp):
+    n = torch.cuda.get_device_properties(0).multi_processor_count // 4
+    q = Problem(256, 2, [(0, 0), (5, 3), (1, 11)], (261, 267))
+    S = 3 * n + 2
+    bad = [0, 1 + n, 2 + 2 * n, 3, 3 + n, 4, 4 + n, 4 + 2 * n]
+    args, (loss, dV, dp), good = q.run(msp, np.arange(S) % 3, bad)
+    el, eV, ep = q.expect(good)
+    assert abs(float(loss) / el - 1) < TOL and rel(dV.cpu(), eV) < TOL and rel(dp.cpu(), ep) < TOL
+    g, probe, V, pos, I = args
+    out = msp.forward(g, probe, V, pos).cpu().numpy()
+    assert float(msp.loss_grad(g, probe, V, pos, I, want_dV=False, want_dprobe=False)[0]) == float(loss)
+    ref = O.forward(q.gd, q.probe, q.windows, V=q.V)
+    for s in (1, 2, 5, n, 2 * n + 3, 3 * n + 1):
+        assert rel(out[s], ref[s % 3]) < TOL
+    for b in bad:
+        assert not out[b].any()
+
+
+@pytest.mark.parametrize("win", [64, 128, 256])
+def test_a_captured_pass_replays_as_it_ran(msp, win):
+    """The kernels of a pass are launched dependent on one another; a graph keeps those edges."""
+    q = Problem(win, 2, [(0, 0), (2, 3)], (win + 5, win + 7))
+    (g, probe, V, pos, I), (loss, dV, dp), _ = q.run(msp, np.arange(2))
+    ws = msp.make_workspace(g)
+    out = [torch.zeros_like(t) for t in (loss, dV, dp)]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        msp.loss_grad(g, probe, V, pos, I, ws=ws, loss=out[0], dV=out[1], dprobe=out[2])
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    for a, b in zip(out, (loss, dV, dp)):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("win", [64, 128, 256])
 @pytest.mark.parametrize("value", [np.inf, np.nan, -1.0, 0.0, 1e-42, 3e38])
 def test_residual_of_one_unusual_intensity(msp, win, value):
     """One count replaced: the loss and the gradient follow sqrt and the quotient as IEEE arithmetic gives them."""
