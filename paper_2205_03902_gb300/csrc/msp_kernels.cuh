@@ -65,6 +65,20 @@ inline cudaError_t launch_following(void (*kernel)(P...), dim3 grid, dim3 block,
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Launches a fused per-position kernel K on `grid` position slots.
+template <typename K>
+cudaError_t launch_position_as(const PosParams& p, int grid, cudaStream_t st) {
+  static bool attr_done[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 64 && !attr_done[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(K::fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::SMEM);
+    if (e != cudaSuccess) return e;
+    attr_done[dev] = true;
+  }
+  return launch_following(K::fn(), dim3(grid * K::CLUSTER), dim3(K::NT), K::SMEM, st, K::CLUSTER, p);
+}
+
 // A compensated FP32 sum (Knuth's two-sum, the rounding errors summed beside the sum): about 48 bits.
 struct Compensated {
   float s = 0.f, e = 0.f;
