@@ -27,6 +27,8 @@
 namespace msp {
 
 cudaError_t launch_position_kernel(int win, int mode, const PosParams& p, int grid, cudaStream_t st);
+bool position_kernel_leaves_positions(int win, int mode, const PosParams& p);
+cudaError_t launch_position_again(int win, int mode, const PosParams& p, int grid, cudaStream_t st);
 int position_slots(int win);
 
 // the precise-forward mode (msp_precise.cu)
@@ -442,7 +444,7 @@ __global__ void __launch_bounds__(1024) prepare_kernel(const float2* __restrict_
       for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
       if (tid == 0) {
         zthr2[0] = tau2 * t;
-        err[0] = 0;
+        err[0] = err[1] = 0;
       }
     }
     return;
@@ -713,7 +715,7 @@ static Workspace layout(const msp_geometry* g, int gcap, char* base) {
   const size_t plane = (size_t)g->obj_ny * g->obj_nx;
   size_t off = 0;
   auto take = [&](size_t bytes) { char* p = base ? base + off : nullptr; off += align256(bytes); return p; };
-  w.err = (int*)take(sizeof(int));
+  w.err = (int*)take(2 * sizeof(int));
   w.scal = (double*)take(16 * sizeof(double));
   w.red = (double*)take(kRedSlots * sizeof(double));
   w.h1 = (float2*)take(W * sizeof(float2));
@@ -726,6 +728,7 @@ static Workspace layout(const msp_geometry* g, int gcap, char* base) {
   w.dprobe_part = (float2*)take((size_t)gcap * WW * sizeof(float2));
   w.dprobe_sum = (float2*)take(WW * sizeof(float2));
   w.loss_part = (double*)take((S > 0 ? S : 1) * loss_slots(g) * sizeof(double));
+  w.again = (uint8_t*)take(S > 0 ? S : 1);
   w.map0 = (float*)take(2 * plane * sizeof(float));   // complex in transmission mode
   w.map1 = (float*)take(plane * sizeof(float));
   w.precise = precise(g) ? (char*)take(precise_extra_bytes(g->precision, (int)W, (int)L, g->obj_ny, g->obj_nx, (int)S))
@@ -803,6 +806,8 @@ static PosParams base_params(const msp_geometry* g, const float* probe, const fl
   p.willum = c.ws.willum;
   p.dprobe_part = c.ws.dprobe_part;
   p.loss_part = c.ws.loss_part;
+  p.again = c.ws.again;
+  p.again_any = c.ws.err + 1;
   p.err = c.ws.err;
   p.zthr2 = c.ws.scal + 5;
   p.L = g->n_slices;
@@ -862,7 +867,12 @@ static msp_status run_position(const msp_geometry* g, int mode, const PosParams&
     if (n > 1) counted((int)(n - 1));   // profiled_launch counted one
     return s;
   }
-  return profiled_launch(c.st, [&] { return launch_position_kernel(g->win, mode, p, c.grid, c.st); });
+  const bool again = position_kernel_leaves_positions(g->win, mode, p);
+  if (again) counted();   // profiled_launch counts one
+  return profiled_launch(c.st, [&] {
+    const cudaError_t e = launch_position_kernel(g->win, mode, p, c.grid, c.st);
+    return again && e == cudaSuccess ? launch_position_again(g->win, mode, p, c.grid, c.st) : e;
+  });
 }
 
 static msp_status reduce_loss(const msp_geometry* g, Call& c, double* extra) {

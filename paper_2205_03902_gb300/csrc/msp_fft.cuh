@@ -139,6 +139,7 @@ template <int W, int T = 8>
 struct RegisterTwiddles {
   float2 r[8];   // r[0] unused (k1 = 0 is never multiplied); r[k] = w^(j k), k = 1..7
   float2 w8;     // w^(8 j)
+  RegisterTwiddles() = default;
   __device__ __forceinline__ RegisterTwiddles(const float2* __restrict__ t, int j) {
 #pragma unroll
     for (int k = 1; k < 8; ++k) r[k] = t[k * T + j];
@@ -202,6 +203,43 @@ __device__ __forceinline__ void line_fft_t(float2 (&v)[W / 8], const Tw& tw, flo
     dft<8, 1>(b[mc], X);
 #pragma unroll
     for (int k2 = 0; k2 < 8; ++k2) v[mc + NC * k2] = INV ? cconj(X[k2]) : X[k2];
+  }
+}
+
+// The same transform of a line held by T threads, exchanged through the line's own W places instead of a buffer
+// beside the wave: load(e) and store(e, x) reach place e.  Operation for operation line_fft_t, so the results have the
+// same bits.  The caller has read the line (the places are free) and stores it back or not.
+template <int K1, int N1, int T, typename Tw, typename Store>
+__device__ __forceinline__ void twiddle_store_in_place(const float2* y, const Tw& tw, const Store& store, int j) {
+  if constexpr (K1 < N1) {
+    store(K1 * T + (j ^ (K1 & (T - 1))), (K1 == 0) ? y[K1] : cmul(y[K1], tw.template get<K1>()));
+    twiddle_store_in_place<K1 + 1, N1, T>(y, tw, store, j);
+  }
+}
+template <int W, int T, bool INV, typename Tw, typename Load, typename Store>
+__device__ __forceinline__ void line_fft_in_place(float2 (&v)[W / T], const Tw& tw, const Load& load, const Store& store, int j) {
+  constexpr int N1 = W / T;
+  constexpr int NC = N1 / T;
+  float2 y[N1], b[NC][T];
+  if constexpr (INV) {
+#pragma unroll
+    for (int m = 0; m < N1; ++m) v[m] = cconj(v[m]);
+  }
+  dft<N1, 1>(v, y);
+  __syncwarp();   // every thread of the group has read its part of the line
+  twiddle_store_in_place<0, N1, T>(y, tw, store, j);
+  __syncwarp();
+#pragma unroll
+  for (int mc = 0; mc < NC; ++mc)
+#pragma unroll
+    for (int n2 = 0; n2 < T; ++n2) b[mc][n2] = load((j + T * mc) * T + (n2 ^ j));
+  __syncwarp();
+#pragma unroll
+  for (int mc = 0; mc < NC; ++mc) {
+    float2 X[T];
+    dft<T, 1>(b[mc], X);
+#pragma unroll
+    for (int k2 = 0; k2 < T; ++k2) v[mc + NC * k2] = INV ? cconj(X[k2]) : X[k2];
   }
 }
 

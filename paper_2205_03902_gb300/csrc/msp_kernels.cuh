@@ -26,7 +26,9 @@ struct PosParams {
                            // order of the additions is not fixed)
   float* illumred;         // [Ny][Nx], zeroed: the layer step's |psi_in,l|^2 likewise, instead of willum
   float2* dprobe_part;     // [G][W][W] per-CTA probe-gradient partial sums
-  double* loss_part;       // [S] per-position loss
+  double* loss_part;       // [S] per-position loss ([S][4], one per CTA, for W = 256)
+  uint8_t* again;          // [S] 1: the position is left to the second launch (W = 128, 256; not forward)
+  int* again_any;          // whether there is such a position
   const double* zthr2;     // [1] squared far-field amplitude that counts as zero
   int* err;                // error flags
   int L, Ny, Nx, S;
@@ -98,7 +100,7 @@ struct Compensated {
 
 // Workspace carve-up (all offsets 256-byte aligned).
 struct Workspace {
-  int* err;
+  int* err;                // [2] window error; whether any `again` is set
   double* scal;            // [16] scalars: 0 loss, 1 mu, 2 max illum, 3 sum I, 5 zero-rule threshold^2
   double* red;             // [kRedSlots] block partials of FP64 reductions, or (as floats) per-tile maxima
   float2* h1;              // [W]
@@ -108,7 +110,8 @@ struct Workspace {
   float* willum;
   float2* dprobe_part;
   float2* dprobe_sum;      // [W][W]
-  double* loss_part;       // [S]
+  double* loss_part;       // [S], or [S][4]
+  uint8_t* again;          // [S] positions left to the second launch of a pass
   float* map0;             // [Ny][Nx] layer gradient map
   float* map1;             // [Ny][Nx] illumination map
   char* precise;           // the precise-forward mode's buffers (NULL in the FP32 mode)

@@ -380,6 +380,8 @@ static cudaError_t launch_64(int mode, const PosParams& p, int grid, cudaStream_
 template <int W>
 cudaError_t launch_wave(int mode, const PosParams& p, int grid, cudaStream_t st);
 template <int W>
+cudaError_t launch_again(int mode, const PosParams& p, int grid, cudaStream_t st);
+template <int W>
 int wave_slots(int sms);
 
 // `grid` counts position slots: CTAs for W = 64 / 128, four-CTA clusters for W = 256.
@@ -388,6 +390,14 @@ cudaError_t launch_position_kernel(int win, int mode, const PosParams& p, int gr
   if (win == 256) return launch_wave<256>(mode, p, grid, st);
   // the forward model reads the slices the same way in both parametrisations
   return p.cplx && mode != MODE_FORWARD ? launch_64<true>(mode, p, grid, st) : launch_64<false>(mode, p, grid, st);
+}
+
+// Whether a pass may leave positions to a second launch (msp_wave.cuh), which has to follow it.
+bool position_kernel_leaves_positions(int win, int mode, const PosParams& p) {
+  return win != 64 && mode != MODE_FORWARD && !p.loss_only;
+}
+cudaError_t launch_position_again(int win, int mode, const PosParams& p, int grid, cudaStream_t st) {
+  return win == 128 ? launch_again<128>(mode, p, grid, st) : launch_again<256>(mode, p, grid, st);
 }
 
 // Positions the fused kernel processes at once on the current device (its persistent grid): resident CTAs for

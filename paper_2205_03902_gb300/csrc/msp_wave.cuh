@@ -42,6 +42,8 @@ constexpr int NT = 512, V = 32;     // threads per CTA, values per thread
 constexpr int CL = 32, RC = 16;     // column n2 extent (lanes), rows' n2 per CTA (warps)
 constexpr int XS = CL + 2;          // row stride of a region (float2): 16-byte accesses of rows are conflict-free
 constexpr int REGION = V * XS;
+constexpr float kBand = 0.1f;       // half width of the band around the zero rule's threshold in |Psi|^2, times sqrt(L)
+constexpr float kJump = 2e-6f;      // the least change of all residuals' norm that a decision is taken again for
 constexpr int TBUF = 16;            // transmission values per thread that are fetched a pass ahead
 constexpr size_t SMEM = ((size_t)RC * REGION + (size_t)TBUF * NT) * sizeof(float2);
 
@@ -121,9 +123,109 @@ __device__ __forceinline__ C2 rotate_back(const C2& v, const float4& w) {
 __device__ __forceinline__ bool word(uint32_t a, uint32_t b) {
   return (anew(a) & b) != 0;
 }
+
+// The zero rule decides by |Psi| > tau ||p||, and R jumps by sqrt(I) there. Two forward models that round differently decide
+// a value near the threshold either way: this kernel and the line transforms differ by 1.3 % of it times sqrt(L)
+// (rms, W = 128 and 256, L = 1 to 16). Where counts were measured, one such decision moves dV by up to 4.5e-5 of its norm
+// (W = 128, L = 4, 1024 positions: two inputs of forty), twenty times what rounding does. So a pass leaves a position with
+// a value within the band (3.9 times that rms) and a jump above kJump of the far fields' norm sqrt(S) W ||p|| to
+// a second launch, which takes the decisions of the whole position from the line transforms, the arithmetic of W = 64:
+// they then depend on the inputs and not on the kernel. At W = 128, L = 4, 1024 positions one pass in five has such a
+// position. Without one the second launch costs 2.2 us (of 672), with one or two 150 us. Deciding within the pass instead
+// was slower throughout: the line transforms' code in this kernel takes registers from all of it (675 -> 715 to 812 us).
+//
+// Which of this thread's far-field values count as nonzero by that arithmetic: bit 2 k + e for value k of column
+// kc + CH e (wave_kernel's pass C).  The forward model once more, every line by a group of 8 (W = 128) or 16 threads
+// that exchanges through the line's own places, the wave in `sm` (W W / RANKS values per CTA).  Called by every
+// thread of the CTA (cluster), when nothing else needs `sm`; it is free again on return.
+template <int W>
+__device__ __noinline__ uint32_t counted_by_lines(const float2* __restrict__ probe, const float2* __restrict__ T, size_t plane,
+                                                  int Nx, int L, float2* sm, const float2* s_w, const float2* s_h1, float zthr2,
+                                                  int rank, int k1r, int kc) {
+  constexpr int RANKS = W == 256 ? 4 : 1, RW = W / RANKS;          // lines per CTA and direction
+  constexpr int TL = W == 128 ? 8 : 16, N1 = W / TL, GROUPS = NT / TL;
+  constexpr int RH = W == 128 ? 8 : 4, CH = W / CL;
+  const int j = threadIdx.x % TL, grp = threadIdx.x / TL;
+  RegisterTwiddles<W, TL> tw;
+#pragma unroll
+  for (int k = 1; k < 8; ++k) tw.r[k] = s_w[k * j];
+  tw.w8 = s_w[8 * j];
+  // value (r, c): row r % RW of CTA r / RW; the permutation spreads rows and columns over the banks
+  auto at = [](int r, int c) { return (r % RW) * W + (c ^ (W == 128 ? swz(r) : r & 15)); };
+  auto load = [&](int r, int c) {
+    if constexpr (RANKS == 1) return sm[at(r, c)];
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr(sm + at(r, c), r / RW)) : "memory");
+    return v;
+  };
+  auto store = [&](int r, int c, float2 v) {
+    if constexpr (RANKS == 1) sm[at(r, c)] = v;
+    else asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(cluster_addr(sm + at(r, c), r / RW)), "f"(v.x), "f"(v.y) : "memory");
+  };
+  auto sync = [] {
+    if constexpr (RANKS == 1) __syncthreads();
+    else cluster_sync();
+  };
+#pragma unroll 1
+  for (int l = 0; l < L; ++l) {
+#pragma unroll 1
+    for (int r = rank * RW + grp; r < (rank + 1) * RW; r += GROUPS) {
+      float2 v[N1];
+      auto get = [&](int e) { return sm[at(r, e)]; };
+      auto put = [&](int e, float2 x) { sm[at(r, e)] = x; };
+      if (l == 0) {
+#pragma unroll
+        for (int m = 0; m < N1; ++m) v[m] = probe[r * W + j + TL * m];
+      } else {
+#pragma unroll
+        for (int m = 0; m < N1; ++m) v[m] = get(j + TL * m);
+        line_fft_in_place<W, TL, true>(v, tw, get, put, j);
+      }
+      const float2* Tr = T + l * plane + (size_t)r * Nx + j;
+#pragma unroll
+      for (int m = 0; m < N1; ++m) v[m] = cmul(v[m], Tr[TL * m]);
+      line_fft_in_place<W, TL, false>(v, tw, get, put, j);
+#pragma unroll
+      for (int m = 0; m < N1; ++m) put(j + TL * m, v[m]);
+    }
+    sync();
+#pragma unroll 1
+    for (int c = rank * RW + grp; c < (rank + 1) * RW; c += GROUPS) {
+      float2 v[N1];
+      auto get = [&](int e) { return load(e, c); };
+      auto put = [&](int e, float2 x) { store(e, c, x); };
+#pragma unroll
+      for (int m = 0; m < N1; ++m) v[m] = get(j + TL * m);
+      line_fft_in_place<W, TL, false>(v, tw, get, put, j);
+      if (l < L - 1) {
+        const float2 hx = s_h1[c];
+#pragma unroll
+        for (int m = 0; m < N1; ++m) v[m] = cmul(v[m], cmul(s_h1[j + TL * m], hx));
+        line_fft_in_place<W, TL, true>(v, tw, get, put, j);
+      } else {
+#pragma unroll
+        for (int m = 0; m < N1; ++m) v[m].x = fmaf(v[m].x, v[m].x, v[m].y * v[m].y);
+      }
+#pragma unroll
+      for (int m = 0; m < N1; ++m) put(j + TL * m, v[m]);
+    }
+    sync();
+  }
+  uint32_t counted = 0;
+#pragma unroll 1
+  for (int k = 0; k < 16; ++k) {
+    const int r = W == 128 ? k1r + RH * k : k1r + RH * (4 * rank + (k >> 2) + 16 * (k & 3));
+#pragma unroll
+    for (int e = 0; e < 2; ++e) counted |= (uint32_t)(load(r, kc + CH * e).x > zthr2) << (2 * k + e);
+  }
+  sync();
+  return counted;
+}
 }  // namespace wave
 
-template <int W, int MODE, bool CPLX>
+// AGAIN: the positions that the pass marked (p.again), with their zero-rule decisions from the line transforms. Usually there
+// is none and the launch ends at once.
+template <int W, int MODE, bool CPLX, bool AGAIN>
 __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
   using namespace wave;
   constexpr bool kCluster = W == 256;
@@ -139,6 +241,7 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
   __shared__ float4 s_hd[W];    // the same, (re, re, im, im)
   __shared__ float red[NT / 32];
   __shared__ float s_zthr2;
+  __shared__ uint32_t s_near[2];   // whether a value of the j-th position lies within the band, in s_near[j & 1]
   __shared__ int2 s_pos[2];     // window origins of this CTA's positions, the j-th one in s_pos[j & 1]
   __shared__ uint32_t s_tmem;
 
@@ -159,6 +262,7 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
   }
   constexpr bool kStash = MODE == MODE_LOSS_GRAD || MODE == MODE_LAYER;
   wait_for_predecessor();
+  if (AGAIN && p.again_any[0] == 0) return;
   if (tid < W) {
     const float2 h = p.h1[tid];
     s_h1[tid] = h;
@@ -171,8 +275,9 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
   }
   if (MODE != MODE_FORWARD && tid == 0) s_zthr2 = (float)p.zthr2[0];
   if (tid < 2) {
+    s_near[tid] = 0;
     const int sp = slot + tid * slots;
-    s_pos[tid] = sp < p.S ? p.pos[sp] : make_int2(-1, -1);
+    s_pos[tid] = !AGAIN && sp < p.S ? p.pos[sp] : make_int2(-1, -1);
   }
   __syncthreads();
   if constexpr (kStash) {
@@ -356,7 +461,7 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
   // registers, and the few that do not fit go to local memory at L2 latency (measured: 722 bytes of spills
   // made the loss-and-gradient pass 1.16 times as long as 230 bytes).
   constexpr uint32_t kFetched = 2, kSummed = 4;
-  uint32_t state = 0;
+  uint32_t state = AGAIN ? kSummed : 0u;
   auto fetch_next_first = [&]() {
     const uint32_t at = window(state + 1);
     if (at != kNoWindow) fetch_first(p.T + (at + (uint32_t)n2 * (uint32_t)p.Nx + (uint32_t)lane));
@@ -373,8 +478,16 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
     if (tid == 0 && sp >= p.S) s_pos[state & 1] = make_int2(-1, -1);
   };
   for (int s = slot; s < p.S; s += slots, state ^= 1) {
+    uint32_t counted = 0;   // AGAIN: the decisions, bit 2 k + e for value k of column e of pass C
+    if constexpr (AGAIN) {
+      if (!p.again[s]) continue;
+      const int2 ps = p.pos[s];   // the slots of the origins stay empty: nothing is fetched for a coming position
+      __syncthreads();
+      if (tid == 0) s_pos[state & 1] = ps;
+      __syncthreads();
+    }
     const uint32_t at = window(state);
-    if (at == kNoWindow) {
+    if (!AGAIN && at == kNoWindow) {
       if (tid == 0) atomicMax(p.err, 1);
       // outputs of a skipped position are zero; each CTA writes its share
       auto zero = [&](auto* a, size_t n) {
@@ -382,7 +495,10 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
       };
       constexpr int CW = CPLX ? 2 : 1;
       if (MODE == MODE_FORWARD) zero(p.I_out + s * WW, WW);
-      if (MODE != MODE_FORWARD && tid == 0) p.loss_part[s * RANKS + rank] = 0.0;
+      if (MODE != MODE_FORWARD && tid == 0) {
+        p.loss_part[s * RANKS + rank] = 0.0;
+        if (rank == 0) p.again[s] = 0;
+      }
       if (MODE == MODE_LOSS_GRAD && !p.dVred && !p.loss_only) zero(p.wgrad + CW * s * WW * L, CW * WW * L);
       if (MODE == MODE_LAYER && !p.dVred) {
         zero(p.wgrad + CW * s * WW, CW * WW);
@@ -399,6 +515,7 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
     const uint32_t oc = at + (uint32_t)n2 * (uint32_t)p.Nx + (uint32_t)lane;   // object offset of this thread's value (0, 0)
     float4* stash = reinterpret_cast<float4*>(p.stash + (size_t)slot * (MODE == MODE_LOSS_GRAD ? L : 1) * WW) + rank * (WW / 2 / RANKS);
     const bool forward_only = MODE == MODE_FORWARD || p.loss_only;
+    if constexpr (AGAIN) counted = counted_by_lines<W>(p.probe, p.T + at, plane, p.Nx, L, sm, s_w, s_h1, s_zthr2, rank, k1r, kc);
     // what the buffer tb receives after slice l's pass on the way forward: the next slice's window, or this
     // thread's values of the measured pattern, or slice 0 of the next position
     auto fetch_after = [&](int l) {
@@ -516,20 +633,26 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
             out[CH] = a2.y;
           }
         } else {   // far field, residual R = Psi - sqrt(I) Psi / |Psi|
-          const float zthr2 = s_zthr2;
+          const float zthr2 = s_zthr2, band = kBand * sqrtf((float)L) * zthr2;
+          const float least = (kJump / (float)kZeroRuleTau) * (kJump / (float)kZeroRuleTau) * (float)p.S * (float)WW * zthr2;
           float lsum = 0.f;
-          bool finite = true;
+          bool finite = true, near = false;
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
             const float2 a2 = fma2(X[k].re, X[k].re, mul2(X[k].im, X[k].im));
             finite = finite && residual_is_finite(a2.x, tb[k * NT].x) && residual_is_finite(a2.y, tb[k * NT].y);
           }
+          auto look = [&](float a2, float I) { near = near || (fabsf(a2 - zthr2) <= band && !(fabsf(I) <= least)); };
+          // the threshold of value 2 k + e
+          auto threshold = [&](int i) { return !AGAIN ? zthr2 : (counted >> i) & 1 ? 0.f : INFINITY; };
           if (finite) {
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
               const float2 a2 = fma2(X[k].re, X[k].re, mul2(X[k].im, X[k].im));
               const float2 im = tb[k * NT];
-              const float2 f = make_float2(residual_finite(a2.x, im.x, zthr2, lsum), residual_finite(a2.y, im.y, zthr2, lsum));
+              const float2 f = make_float2(residual_finite(a2.x, im.x, threshold(2 * k), lsum), residual_finite(a2.y, im.y, threshold(2 * k + 1), lsum));
+              look(a2.x, im.x);
+              look(a2.y, im.y);
               X[k] = {mul2(X[k].re, f), mul2(X[k].im, f)};
             }
           } else if (kCluster) {   // the slots of the wave are still being read by the other CTAs
@@ -537,7 +660,9 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
             for (int k = 0; k < 16; ++k) {
               const float2 a2 = fma2(X[k].re, X[k].re, mul2(X[k].im, X[k].im));
               const float2 im = tb[k * NT];
-              const float2 f = make_float2(residual_exact(a2.x, im.x, zthr2, lsum), residual_exact(a2.y, im.y, zthr2, lsum));
+              const float2 f = make_float2(residual_exact(a2.x, im.x, threshold(2 * k), lsum), residual_exact(a2.y, im.y, threshold(2 * k + 1), lsum));
+              look(a2.x, im.x);
+              look(a2.y, im.y);
               X[k] = {mul2(X[k].re, f), mul2(X[k].im, f)};
             }
           } else {   // through this thread's slots of the wave, to keep the rare path short
@@ -548,14 +673,24 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
             for (int k = 0; k < 16; ++k) {
               float4& f = *reinterpret_cast<float4*>(sc + k * REGION);
               const float2 im = tb[k * NT];
-              const float fx = residual_exact(fmaf(f.x, f.x, f.z * f.z), im.x, zthr2, lsum);
-              const float fy = residual_exact(fmaf(f.y, f.y, f.w * f.w), im.y, zthr2, lsum);
+              look(fmaf(f.x, f.x, f.z * f.z), im.x);
+              look(fmaf(f.y, f.y, f.w * f.w), im.y);
+              const float fx = residual_exact(fmaf(f.x, f.x, f.z * f.z), im.x, threshold(2 * k), lsum);
+              const float fy = residual_exact(fmaf(f.y, f.y, f.w * f.w), im.y, threshold(2 * k + 1), lsum);
               f = make_float4(f.x * fx, f.y * fy, f.z * fx, f.w * fy);
             }
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
               const float4 f = *reinterpret_cast<const float4*>(sc + k * REGION);
               X[k] = {make_float2(f.x, f.y), make_float2(f.z, f.w)};
+            }
+          }
+          if (!AGAIN && near && !p.loss_only) {   // the position is left to the launch that decides
+            if constexpr (kCluster) {
+              for (int r = 0; r < RANKS; ++r)
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(&s_near[state & 1], r)), "r"(1) : "memory");
+            } else {
+              s_near[state & 1] = 1;
             }
           }
 #pragma unroll
@@ -587,24 +722,40 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
       if (kCluster && st == L - 1 && forward_only) cluster_sync();   // the other CTAs have read this one's regions
       else __syncthreads();
       if (st == L - 1) {
+        bool ends = forward_only;   // no adjoint
+        if (!AGAIN && MODE != MODE_FORWARD) {
+          const uint32_t left = s_near[state & 1];
+          ends = ends || left;
+          if (tid == 0) {
+            s_near[~state & 1] = 0;   // the coming position's; nobody looks at it before another barrier
+            if (rank == 0) {
+              p.again[s] = left;
+              if (left) p.again_any[0] = 1;
+            }
+          }
+        }
         // the pattern has been read: the buffer takes the last slice's window again, or the next position's first
         if (MODE != MODE_FORWARD) {
-          if (!p.loss_only) fetch_first(p.T + (size_t)(L - 1) * plane + oc);
+          if (!ends) fetch_first(p.T + (size_t)(L - 1) * plane + oc);
           else fetch_next_first();
         }
         if (MODE == MODE_FORWARD && L == 1) fetch_next_first();
-        if (forward_only) fetch_next_second();
+        if (ends) fetch_next_second();
         state = (state & ~kFetched) | (window(state + 1) != kNoWindow ? kFetched : 0u);
-        fetch_origin(s);
+        if (AGAIN) {
+          if (tid == 0) s_pos[state & 1] = make_int2(-1, -1);
+        } else {
+          fetch_origin(s);
+        }
         fetch_commit();
         if (MODE == MODE_FORWARD) break;
-        if (tid == 0) {
+        if (!AGAIN && tid == 0) {   // the pass itself has summed the loss
           double acc = 0.0;
 #pragma unroll 1
           for (int w = 0; w < NT / 32; ++w) acc += (double)red[w];
           p.loss_part[s * RANKS + rank] = acc;
         }
-        if (p.loss_only) break;
+        if (ends) break;
       }
       {   // ---------------- inverse pass B ----------------
         float4* q = reinterpret_cast<float4*>(sb);
@@ -718,11 +869,11 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
 // ----------------------------------------------------------------------------
 // launch helpers
 // ----------------------------------------------------------------------------
-template <int W, int MODE, bool CPLX>
+template <int W, int MODE, bool CPLX, bool AGAIN = false>
 struct WaveKernel {
   static constexpr int NT = wave::NT, CLUSTER = W == 256 ? 4 : 1;
   static constexpr size_t SMEM = wave::SMEM;
-  static void (*fn())(const PosParams) { return wave_kernel<W, MODE, CPLX>; }
+  static void (*fn())(const PosParams) { return wave_kernel<W, MODE, CPLX, AGAIN>; }
 };
 
 template <int W, bool CPLX>
@@ -739,6 +890,20 @@ cudaError_t launch_wave(int mode, const PosParams& p, int grid, cudaStream_t st)
   // the forward model reads the slices the same way in both parametrisations
   if (p.cplx && mode != MODE_FORWARD) return launch_wave_of<W, true>(mode, p, grid, st);
   return launch_wave_of<W, false>(mode, p, grid, st);
+}
+
+// The positions of a pass just launched that it left to the line transforms.
+template <int W, bool CPLX>
+static cudaError_t launch_again_of(int mode, const PosParams& p, int grid, cudaStream_t st) {
+  switch (mode) {
+    case MODE_LOSS_GRAD: return launch_position_as<WaveKernel<W, MODE_LOSS_GRAD, CPLX, true>>(p, grid, st);
+    case MODE_LAYER: return launch_position_as<WaveKernel<W, MODE_LAYER, CPLX, true>>(p, grid, st);
+    default: return launch_position_as<WaveKernel<W, MODE_PROBE, CPLX, true>>(p, grid, st);
+  }
+}
+template <int W>
+cudaError_t launch_again(int mode, const PosParams& p, int grid, cudaStream_t st) {
+  return p.cplx ? launch_again_of<W, true>(mode, p, grid, st) : launch_again_of<W, false>(mode, p, grid, st);
 }
 
 // Positions that are resident at once on this device: one per CTA of 512 threads (W = 128), or per four-CTA cluster.

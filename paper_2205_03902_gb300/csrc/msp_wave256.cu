@@ -4,6 +4,7 @@
 namespace msp {
 
 template cudaError_t launch_wave<256>(int mode, const PosParams& p, int grid, cudaStream_t st);
+template cudaError_t launch_again<256>(int mode, const PosParams& p, int grid, cudaStream_t st);
 template int wave_slots<256>(int sms);
 
 }  // namespace msp
