@@ -320,9 +320,8 @@ __global__ void __launch_bounds__(256) sum_blocks_kernel(const float* __restrict
 // dprobe[i] = sum_b part[b][i], fixed order.  A block of 256 threads owns 32 consecutive probe values: warp g
 // sums the partials b = g, g + 8, g + 16, ... (lane = value, so every load is 256 contiguous bytes), all of
 // them in flight at once, and the eight warp sums are added in warp order.  512 blocks for W = 128 keep
-// every SM loading.  The sums are compensated (Knuth's two-sum, the rounding errors summed beside the sum):
-// about 48 bits before the one rounding to FP32, the same results as FP64 sums, whose additions and
-// conversions at 1/64 of the FP32 rate took most of the time (64 partials of W = 64: 10.7 us).
+// every SM loading.  The sums are FP64's to the bit, in compensated FP32: FP64 additions and conversions at 1/64 of the
+// FP32 rate took most of the time (64 partials of W = 64: 10.7 us).
 constexpr int kDprobeVals = 32;
 // the sum of value blk kDprobeVals + lane, in the lanes of warp 0
 __device__ __forceinline__ float2 dprobe_sum(const float2* __restrict__ part, int G, int WW, int blk) {
@@ -354,7 +353,7 @@ __device__ __forceinline__ float2 dprobe_sum(const float2* __restrict__ part, in
     re.add(acc_w[w][lane][0]);
     im.add(acc_w[w][lane][1]);
   }
-  return make_float2(re.value(), im.value());
+  return make_float2((float)re.wide(), (float)im.wide());
 }
 __device__ __forceinline__ void dprobe_block(const float2* __restrict__ part, int G, int WW, float2* __restrict__ out,
                                              int blk) {

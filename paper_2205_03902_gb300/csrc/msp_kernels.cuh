@@ -81,21 +81,27 @@ cudaError_t launch_position_as(const PosParams& p, int grid, cudaStream_t st) {
   return launch_following(K::fn(), dim3(grid * K::CLUSTER), dim3(K::NT), K::SMEM, st, K::CLUSTER, p);
 }
 
-// A compensated FP32 sum (Knuth's two-sum, the rounding errors summed beside the sum): about 48 bits.
+// An FP64 sum of FP32 values without the FP64 pipe, which converts and adds about one value per cycle and SM: three
+// FP32 terms, the sum, its rounding errors (Knuth's two-sum) and theirs (cascaded, Klein 2006), about 72 bits before the one
+// rounding to FP64. A sum that leaves FP32's range is not finite, and the caller takes it again in FP64.
 struct Compensated {
-  float s = 0.f, e = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float t = s + v, b = t - s;
-    e += (s - (t - b)) + (v - b);
-    s = t;
+  float s = 0.f, e = 0.f, ee = 0.f;
+  // x + v in x, returns the rounding error
+  static __device__ __forceinline__ float two_sum(float& x, float v) {
+    const float t = x + v, b = t - x;
+    const float r = (x - (t - b)) + (v - b);
+    x = t;
+    return r;
   }
+  __device__ __forceinline__ void add_error(float v) { ee += two_sum(e, v); }
+  __device__ __forceinline__ void add(float v) { add_error(two_sum(s, v)); }
   __device__ __forceinline__ void add(const Compensated& c) {
     add(c.s);
-    e += c.e;
+    add_error(c.e);
+    ee += c.ee;
   }
-  // e is NaN where s is not finite
-  __device__ __forceinline__ float value() const { return e == e ? s + e : s; }
-  __device__ __forceinline__ double wide() const { return e == e ? (double)s + (double)e : (double)s; }
+  // where s is not finite, its errors are NaN
+  __device__ __forceinline__ double wide() const { return ee == ee ? (double)s + ((double)e + (double)ee) : (double)s; }
 };
 
 // Workspace carve-up (all offsets 256-byte aligned).

@@ -654,7 +654,7 @@ __global__ void output_kernel(const float* __restrict__ pre, int L, size_t P, fl
 // pre-activation (bf16 NHWC, padded channels 0); per-block loss partials (FP64).
 // One thread per pixel: its 16 channels are four 16-byte loads and two 16-byte stores, the target's planes are read in
 // rows.  A thread sums its squares in compensated FP32, rounding errors of the products included, and a pixel whose
-// sum leaves the range where these are exact to 1e-13 again in FP64: in FP64 alone, whose pipe takes about one
+// sum leaves the range where these are exact to FP64's rounding again in FP64: in FP64 alone, whose pipe takes about one
 // conversion or addition per cycle and SM, the kernel took 19 us at 384 x 384 with either split; it takes 9.5.
 __global__ void __launch_bounds__(256) loss_kernel(const float* __restrict__ pre, const float* __restrict__ target, int L,
                                                    size_t P, float inv_sd, bf16* __restrict__ g,
@@ -680,7 +680,7 @@ __global__ void __launch_bounds__(256) loss_kernel(const float* __restrict__ pre
       const float d = c < L ? x[c] - inv_sd * y[c] : 0.f;
       const float d2 = d * d;
       pixel.add(d2);
-      pixel.e += fmaf(d, d, -d2);
+      pixel.add_error(fmaf(d, d, -d2));
       x[c] = d;
       o[c] = __float2bfloat16_rn(c < L ? scale * d : 0.f);
     }

@@ -742,7 +742,7 @@ __global__ void __launch_bounds__(32 * kGroups) grad_step_kernel(float2* __restr
                                                         const double* __restrict__ obj_part,
                                                         double* __restrict__ normpart, double* scal,
                                                         double* obj_out) {
-  __shared__ float4 sh[kGroups][32];   // (re.s, re.e, im.s, im.e)
+  __shared__ Compensated sh[kGroups][2][32];
   __shared__ double red[32 * kGroups + 1];
   __shared__ double maxo[kMaxSlices];
   const int t = threadIdx.x, lane = t & 31, grp = t >> 5;
@@ -764,7 +764,8 @@ __global__ void __launch_bounds__(32 * kGroups) grad_step_kernel(float2* __restr
       re.add(v.x);
       im.add(v.y);
     }
-  sh[grp][lane] = make_float4(re.s, re.e, im.s, im.e);
+  sh[grp][0][lane] = re;
+  sh[grp][1][lane] = im;
   __syncthreads();
   if (grp == 0) {
     double2 g;
@@ -772,9 +773,8 @@ __global__ void __launch_bounds__(32 * kGroups) grad_step_kernel(float2* __restr
       g = make_double2(g0[k].x, g0[k].y);
     } else {
       for (int q = 1; q < kGroups; ++q) {
-        const float4 v = sh[q][lane];
-        re.add(Compensated{v.x, v.y});
-        im.add(Compensated{v.z, v.w});
+        re.add(sh[q][0][lane]);
+        im.add(sh[q][1][lane]);
       }
       g = make_double2(re.wide(), im.wide());
       if (!isfinite(g.x) || !isfinite(g.y)) {   // a partial, or only its FP32 sum: FP64 tells
