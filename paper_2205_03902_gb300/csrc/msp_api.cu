@@ -353,7 +353,16 @@ __device__ __forceinline__ float2 dprobe_sum(const float2* __restrict__ part, in
     re.add(acc_w[w][lane][0]);
     im.add(acc_w[w][lane][1]);
   }
-  return make_float2((float)re.wide(), (float)im.wide());
+  double2 t = make_double2(re.wide(), im.wide());
+  if ((!isfinite(t.x) || !isfinite(t.y)) && i < WW) {   // a partial, or only a sum in FP32's range: FP64 tells
+    t = make_double2(0.0, 0.0);
+    for (int b = 0; b < G; ++b) {
+      const float2 v = part[(size_t)b * WW + i];
+      t.x += v.x;
+      t.y += v.y;
+    }
+  }
+  return make_float2((float)t.x, (float)t.y);
 }
 __device__ __forceinline__ void dprobe_block(const float2* __restrict__ part, int G, int WW, float2* __restrict__ out,
                                              int blk) {

@@ -707,8 +707,17 @@ __global__ void __launch_bounds__(64) dprobe_accumulate_kernel(const float2* __r
       y.add(v[u].y);
     }
   }
+  double2 t = make_double2(x.wide(), y.wide());
+  if (!isfinite(t.x) || !isfinite(t.y)) {   // a term, or only a sum in FP32's range: FP64 tells
+    t = make_double2(0.0, 0.0);
+    for (int b = 0; b < nb; ++b) {
+      const float2 v = contrib[(size_t)b * WW + k];
+      t.x += v.x;
+      t.y += v.y;
+    }
+  }
   const double2 a = first ? make_double2(0.0, 0.0) : dp64[k];
-  dp64[k] = make_double2(a.x + x.wide(), a.y + y.wide());
+  dp64[k] = make_double2(a.x + t.x, a.y + t.y);
 }
 __global__ void dprobe_finish_kernel(const double2* __restrict__ dp64, int WW, float2* __restrict__ out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;

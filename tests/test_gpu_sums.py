@@ -52,6 +52,17 @@ def test_probe_gradient_keeps_the_53rd_bit_of_a_sum(msp, win, precision):
     assert torch.equal(dprobe(msp, win, precision, terms), only(win, win * win * 2.0 ** -52))
 
 
+@pytest.mark.parametrize("win,precision", FORMS)
+def test_probe_gradient_of_a_sum_beyond_single_precision(msp, win, precision):
+    # four times 2^126 and back: the sum reaches 2^128 in between
+    a = 2.0 ** 63 / win
+    terms = [(a, 0.0)] * 4 + [(a, 2.0)] * 4
+    assert torch.equal(dprobe(msp, win, precision, terms), only(win, 0.0))
+    assert torch.equal(dprobe(msp, win, precision, terms[:5]), only(win, 3 * 2.0 ** 126))
+    # a partial that is not finite stays so
+    assert not torch.isfinite(dprobe(msp, win, precision, [(2.0 ** 65 / win, 0.0), (1.0, 0.0)])[0, 0].real)
+
+
 @pytest.mark.parametrize("L", [1, 6, 8])
 def test_training_loss_of_equal_squares(msp, L):
     # the value whose squares' rounding errors add up most in sums of 48 bits: 2.1e-14 at eight channels
