@@ -86,10 +86,10 @@ cudaError_t launch_position_as(const PosParams& p, int grid, cudaStream_t st) {
 // rounding to FP64. A sum that leaves FP32's range is not finite, and the caller takes it again in FP64.
 struct Compensated {
   float s = 0.f, e = 0.f, ee = 0.f;
-  // x + v in x, returns the rounding error
+  // x + v in x, returns the rounding error; the intrinsics are never fused with the product that v may be
   static __device__ __forceinline__ float two_sum(float& x, float v) {
-    const float t = x + v, b = t - x;
-    const float r = (x - (t - b)) + (v - b);
+    const float t = __fadd_rn(x, v), b = __fsub_rn(t, x);
+    const float r = __fadd_rn(__fsub_rn(x, __fsub_rn(t, b)), __fsub_rn(v, b));
     x = t;
     return r;
   }

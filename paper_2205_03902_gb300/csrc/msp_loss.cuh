@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(256) loss_kernel(const float* __restrict__ pre
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
       const float d = c < L ? x[c] - inv_sd * y[c] : 0.f;
-      const float d2 = d * d;
+      const float d2 = __fmul_rn(d, d);   // rounded here: its error is added beside it
       pixel.add(d2);
       pixel.add_error(fmaf(d, d, -d2));
       x[c] = d;
