@@ -23,6 +23,7 @@
 // conflicts for 8-byte elements.
 #pragma once
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace msp {
 
@@ -254,12 +255,13 @@ __device__ __forceinline__ float residual_exact(float a2, float I, float zthr2, 
   lsum = fmaf(d, d, lsum);
   return (a2 > zthr2) ? (1.f - rt / a) : 1.f;   // a2 > zthr2 >= 0 implies a > 0
 }
-// The same for finite a2 and finite I >= 0 without a branch: zero counts are the usual case in a pattern, and
+// The same for a2 and I in range (residual_in_range) without a branch: zero counts are the usual case in a pattern, and
 // the library's square root and quotient leave their short path for zero operands (measured: of 165
 // thousand cycles per position, W = 128, L = 4, 19 went into this pass; W = 64, L = 5, 2115 positions,
 // loss and gradients: 398 -> 383 us).  sqrt(x) = s + (x - s s) y / 2 and n / a = q + (n - q a) y from the
-// reciprocal square root y, with one fused residual each (Markstein 1990).
-__device__ __forceinline__ float residual_finite(float a2, float I, float zthr2, float& lsum) {
+// reciprocal square root y, with one fused residual each (Markstein 1990): the residuals are exact, so each result is
+// within half an ulp but for ties (tests/test_gpu_device_functions.py).
+__device__ __forceinline__ float residual_fast(float a2, float I, float zthr2, float& lsum) {
   const float y = rsqrtf(a2), z = rsqrtf(I);
   float a = a2 * y, rt = I * z;
   a = fmaf(fmaf(-a, a, a2), 0.5f * y, a);
@@ -272,20 +274,22 @@ __device__ __forceinline__ float residual_finite(float a2, float I, float zthr2,
   q = fmaf(fmaf(-q, a, rt), y, q);
   return a2 > zthr2 ? 1.f - q : 1.f;
 }
-__device__ __forceinline__ bool residual_is_finite(float a2, float I) {
-  return a2 <= 3.402823466e+38f && I >= 0.f && I <= 3.402823466e+38f;
+// 2^-100 <= a2 < infinity (below, the residuals' last bits and the quotient leave FP32's range) and 0 <= I < infinity
+__device__ __forceinline__ bool residual_in_range(float a2, float I) {
+  constexpr uint32_t least = 27u << 23, infinity = 255u << 23;
+  return __float_as_uint(a2) - least < infinity - least && I >= 0.f && I <= 3.402823466e+38f;
 }
 
 // v <- f v for N far-field values of a thread and their measured intensities.
 template <int N>
 __device__ __forceinline__ void residual(float2 (&v)[N], const float (&I)[N], float zthr2, float& lsum) {
-  bool finite = true;
+  bool in_range = true;
 #pragma unroll
-  for (int m = 0; m < N; ++m) finite = finite && residual_is_finite(fmaf(v[m].x, v[m].x, v[m].y * v[m].y), I[m]);
+  for (int m = 0; m < N; ++m) in_range = in_range && residual_in_range(fmaf(v[m].x, v[m].x, v[m].y * v[m].y), I[m]);
 #pragma unroll
   for (int m = 0; m < N; ++m) {
     const float a2 = fmaf(v[m].x, v[m].x, v[m].y * v[m].y);
-    const float f = finite ? residual_finite(a2, I[m], zthr2, lsum) : residual_exact(a2, I[m], zthr2, lsum);
+    const float f = in_range ? residual_fast(a2, I[m], zthr2, lsum) : residual_exact(a2, I[m], zthr2, lsum);
     v[m] = make_float2(v[m].x * f, v[m].y * f);
   }
 }

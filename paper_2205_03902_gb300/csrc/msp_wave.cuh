@@ -636,21 +636,21 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
           const float zthr2 = s_zthr2, band = kBand * sqrtf((float)L) * zthr2;
           const float least = (kJump / (float)kZeroRuleTau) * (kJump / (float)kZeroRuleTau) * (float)p.S * (float)WW * zthr2;
           float lsum = 0.f;
-          bool finite = true, near = false;
+          bool in_range = true, near = false;
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
             const float2 a2 = fma2(X[k].re, X[k].re, mul2(X[k].im, X[k].im));
-            finite = finite && residual_is_finite(a2.x, tb[k * NT].x) && residual_is_finite(a2.y, tb[k * NT].y);
+            in_range = in_range && residual_in_range(a2.x, tb[k * NT].x) && residual_in_range(a2.y, tb[k * NT].y);
           }
           auto look = [&](float a2, float I) { near = near || (fabsf(a2 - zthr2) <= band && !(fabsf(I) <= least)); };
           // the threshold of value 2 k + e
           auto threshold = [&](int i) { return !AGAIN ? zthr2 : (counted >> i) & 1 ? 0.f : INFINITY; };
-          if (finite) {
+          if (in_range) {
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
               const float2 a2 = fma2(X[k].re, X[k].re, mul2(X[k].im, X[k].im));
               const float2 im = tb[k * NT];
-              const float2 f = make_float2(residual_finite(a2.x, im.x, threshold(2 * k), lsum), residual_finite(a2.y, im.y, threshold(2 * k + 1), lsum));
+              const float2 f = make_float2(residual_fast(a2.x, im.x, threshold(2 * k), lsum), residual_fast(a2.y, im.y, threshold(2 * k + 1), lsum));
               look(a2.x, im.x);
               look(a2.y, im.y);
               X[k] = {mul2(X[k].re, f), mul2(X[k].im, f)};
