@@ -833,9 +833,9 @@ __global__ void __launch_bounds__(512, 1) wave_kernel(const PosParams p) {
             if (!word(state, kSummed)) {
               d[0] = a;
               d[EW] = b;
-            } else {
-              atomicAdd(d, a);
-              atomicAdd(d + EW, b);
+            } else {   // (a reduction in L2 would flush subnormal sums)
+              d[0] = cadd(d[0], a);
+              d[EW] = cadd(d[EW], b);
             }
           }
         }

@@ -63,6 +63,20 @@ def test_probe_gradient_of_a_sum_beyond_single_precision(msp, win, precision):
     assert not torch.isfinite(dprobe(msp, win, precision, [(2.0 ** 65 / win, 0.0), (1.0, 0.0)])[0, 0].real)
 
 
+@pytest.mark.parametrize("win", [64, 128, 256])
+def test_probe_gradient_keeps_subnormal_contributions(msp, win):
+    # every position on one window, several in each slot of the grid: their own sum is a subnormal FP32 value
+    S = 2 * 2 * torch.cuda.get_device_properties(0).multi_processor_count + 3
+    a = 2.0 ** -70 / win   # a^2 W^2 = 2^-140
+    g = msp.geometry(n_slices=1, obj_ny=win, obj_nx=win, win=win, n_pos=S, wavelength_A=0.0698, sigma=1.5e-3, dz_A=2.0,
+                     pixel_A=0.15, param=msp.MSP_PARAM_TRANSMISSION)
+    T = torch.full((1, win, win), a, dtype=torch.complex64, device="cuda")
+    probe = torch.zeros((win, win), dtype=torch.complex64, device="cuda")
+    probe[0, 0] = 1.0
+    pos, I = torch.zeros((S, 2), dtype=torch.int32, device="cuda"), torch.zeros((S, win, win), device="cuda")
+    assert torch.equal(msp.loss_grad(g, probe, T, pos, I)[2].cpu(), only(win, S * 2.0 ** -140))
+
+
 @pytest.mark.parametrize("L", [1, 6, 8])
 def test_training_loss_of_equal_squares(msp, L):
     # the value whose squares' rounding errors add up most in sums of 48 bits: 2.1e-14 at eight channels
