@@ -79,12 +79,19 @@ def test_residual_of_a_far_field_value(lib, kind):
     assert (np.abs(d - e) <= u * (a + rt)[fits] + 2 * u * e + 2.0 ** -74).all()   # a square below 2^-148 is lost
 
 
+def test_residual_of_a_far_field_value_of_zero(lib):
+    I = np.concatenate([np.arange(4097.0), 10.0 ** np.linspace(-25, 37, 1000)])
+    out = residual(lib, np.zeros(I.size), I, thr2=1e-10).astype(np.float64)
+    assert (out[:, 0] == 1.0).all()
+    assert (np.abs(out[:, 1] - I.astype(np.float32)) <= 3 * 2.0 ** -24 * 1.001 * I).all()   # the root, rounded once, squared
+
+
 def test_residual_of_operands_out_of_range(lib):
     tiny = np.array([0.0, 1e-45, 1e-44, 1e-38, 7e-31, np.inf, np.nan])
     I = np.array([0.0, 1e-45, 1.0, 3e38, np.inf, np.nan, -1.0])
     a2, I = (x.ravel() for x in np.meshgrid(np.concatenate([tiny, [1.0, 3e38]]), I, indexing="ij"))
     for thr2 in (0.0, 1e-40, 1e-3):
         got, want = residual(lib, a2, I, thr2), residual(lib, a2, I, thr2, general=1)
-        out = ~((a2 >= 2.0 ** -100) & (a2 < np.inf) & (I >= 0) & (I < np.inf))
+        out = ~(((a2 == 0) | (a2 >= 2.0 ** -100)) & (a2 < np.inf) & (I >= 0) & (I < np.inf))
         assert np.array_equal(got[out], want[out], equal_nan=True)
         assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
