@@ -1020,7 +1020,7 @@ def run_msp(args, rank, world, local_rank):
     kname = f"position_kernel<{W}, LOSS_GRAD>" if W == 64 else f"wave_kernel<{W}, LOSS_GRAD>"
     traffic = None
     if cfg is synth.C2:
-        traffic = measured_traffic("position_kernel_loss_grad" + ("_l2_reduce" if args.overlap_add == "l2" else ""))
+        traffic = measured_traffic("wave_kernel_loss_grad" + ("_l2_reduce" if args.overlap_add == "l2" else ""))
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",

@@ -378,8 +378,8 @@ __device__ __forceinline__ float2 axpy(float m, float2 u, float2 e) {
 
 // The butterfly e + w o, e - w o with w = exp(-2 pi i K / N) (INV: conjugated), 0 <= K < N / 2, on one
 // complex value (float2) or two (C2).  w is applied as its larger component times (1, tan) or (cot, 1),
-// |tan|, |cot| <= 1: two fused multiply-adds for the rotation and four that scale and add, six
-// operations where a complex product and two sums take eight, with no more roundings on the way.
+// |tan|, |cot| <= 1 (Linzer and Feig, IEEE Trans. Signal Process. 1993): two fused multiply-adds for the rotation and
+// four that scale and add, six operations where a complex product and two sums take eight, with no more roundings on the way.
 template <int N, int K, bool INV, typename T>
 __device__ __forceinline__ void butterfly(T e, T o, T& x0, T& x1) {
   if constexpr (K == 0) {

@@ -29,14 +29,15 @@ namespace msp {
 // writes back to the addresses that it read.  Spectra stay in the order of the split: the propagator and
 // the patterns are indexed by k, and the inverse consumes the same order.
 //
-// Against line transforms by thread groups with an exchange inside each (the form above), a propagation at
+// Against line transforms by thread groups with an exchange inside each (the form of W = 64), a propagation at
 // W = 128 moves the wave through shared memory four times in and out instead of six, and packed arithmetic
-// needs 313 thousand warp instructions per position (L = 4) instead of 441.  What bounds it: the L1 data
-// pipe (61 %), the FP32 pipe (48 %) and issue (46 %) together, with the warps of a position in step between
-// two barriers.  Loss and gradients, W = 128, L = 4, 1024 positions: 0.709 -> 0.59 ms; forward model
-// 0.302 -> 0.251 ms; L = 8, 4096 positions: 5.68 -> 4.77 ms.  W = 256 (L = 16, 2304 positions): 52.5 -> 42.3 ms against
-// rows of the wave per CTA and columns read across the cluster in 8-byte accesses 2 KB apart; the cluster's
-// barriers and the trip through distributed shared memory remain its largest cost.
+// needs 320 thousand warp instructions per position (L = 4) instead of 441.  What bounds it: the L1 data
+// pipe (61 %), the FP32 pipe (51 %) and issue (44 %) together, with the warps of a position in step between
+// two barriers.  Loss and gradients, W = 128, L = 4, 1024 positions: 0.709 -> 0.598 ms; forward model
+// 0.302 -> 0.251 ms.  W = 256 against rows of the wave per CTA and columns read across the cluster in 8-byte accesses
+// 2 KB apart (L = 16, 2304 positions, the whole call): 55.5 -> 44.9 ms.  It issues in 27 % of the cycles; its warps wait
+// for loads from other CTAs' shared memory and the stash (long scoreboard 2.2 of 14.6 cycles per issue, queue for
+// them 2.1), for shared memory (MIO 1.7, short scoreboard 1.4) and at the CTA's and the cluster's barriers (1.2 and 0.9).
 namespace wave {
 constexpr int NT = 512, V = 32;     // threads per CTA, values per thread
 constexpr int CL = 32, RC = 16;     // column n2 extent (lanes), rows' n2 per CTA (warps)
