@@ -171,9 +171,12 @@ __device__ __noinline__ uint32_t counted_by_lines(const float2* __restrict__ pro
   for (int l = 0; l < L; ++l) {
 #pragma unroll 1
     for (int r = rank * RW + grp; r < (rank + 1) * RW; r += GROUPS) {
-      float2 v[N1];
+      float2 v[N1], t[N1];
       auto get = [&](int e) { return sm[at(r, e)]; };
       auto put = [&](int e, float2 x) { sm[at(r, e)] = x; };
+      const float2* Tr = T + l * plane + (size_t)r * Nx + j;
+#pragma unroll
+      for (int m = 0; m < N1; ++m) t[m] = Tr[TL * m];   // in flight during the transform
       if (l == 0) {
 #pragma unroll
         for (int m = 0; m < N1; ++m) v[m] = probe[r * W + j + TL * m];
@@ -182,9 +185,8 @@ __device__ __noinline__ uint32_t counted_by_lines(const float2* __restrict__ pro
         for (int m = 0; m < N1; ++m) v[m] = get(j + TL * m);
         line_fft_in_place<W, TL, true>(v, tw, get, put, j);
       }
-      const float2* Tr = T + l * plane + (size_t)r * Nx + j;
 #pragma unroll
-      for (int m = 0; m < N1; ++m) v[m] = cmul(v[m], Tr[TL * m]);
+      for (int m = 0; m < N1; ++m) v[m] = cmul(v[m], t[m]);
       line_fft_in_place<W, TL, false>(v, tw, get, put, j);
 #pragma unroll
       for (int m = 0; m < N1; ++m) put(j + TL * m, v[m]);
