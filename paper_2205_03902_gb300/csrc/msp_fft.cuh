@@ -207,18 +207,18 @@ __device__ __forceinline__ void line_fft_t(float2 (&v)[W / 8], const Tw& tw, flo
   }
 }
 
-// The same transform of a line held by T threads, exchanged through the line's own W places instead of a buffer
-// beside the wave: load(e) and store(e, x) reach place e.  Operation for operation line_fft_t, so the results have the
-// same bits.  The caller has read the line (the places are free) and stores it back or not.
-template <int K1, int N1, int T, typename Tw, typename Store>
-__device__ __forceinline__ void twiddle_store_in_place(const float2* y, const Tw& tw, const Store& store, int j) {
+// The same transform of a line held by T threads (8 or 16), exchanged through W places at `xb`, in an order that is free of
+// bank conflicts within a warp (`odd`: 1 in every second group of eight). Operation for operation line_fft_t, so the results
+// have the same bits.
+template <int K1, int N1, int T, typename Tw>
+__device__ __forceinline__ void twiddle_store_permuted(const float2* y, const Tw& tw, float2* xb, int j, int odd) {
   if constexpr (K1 < N1) {
-    store(K1 * T + (j ^ (K1 & (T - 1))), (K1 == 0) ? y[K1] : cmul(y[K1], tw.template get<K1>()));
-    twiddle_store_in_place<K1 + 1, N1, T>(y, tw, store, j);
+    xb[(K1 ^ odd) * T + (j ^ (K1 & (T - 1)))] = (K1 == 0) ? y[K1] : cmul(y[K1], tw.template get<K1>());
+    twiddle_store_permuted<K1 + 1, N1, T>(y, tw, xb, j, odd);
   }
 }
-template <int W, int T, bool INV, typename Tw, typename Load, typename Store>
-__device__ __forceinline__ void line_fft_in_place(float2 (&v)[W / T], const Tw& tw, const Load& load, const Store& store, int j) {
+template <int W, int T, bool INV, typename Tw>
+__device__ __forceinline__ void line_fft_permuted(float2 (&v)[W / T], const Tw& tw, float2* xb, int j, int odd) {
   constexpr int N1 = W / T;
   constexpr int NC = N1 / T;
   float2 y[N1], b[NC][T];
@@ -227,14 +227,13 @@ __device__ __forceinline__ void line_fft_in_place(float2 (&v)[W / T], const Tw& 
     for (int m = 0; m < N1; ++m) v[m] = cconj(v[m]);
   }
   dft<N1, 1>(v, y);
-  __syncwarp();   // every thread of the group has read its part of the line
-  twiddle_store_in_place<0, N1, T>(y, tw, store, j);
+  twiddle_store_permuted<0, N1, T>(y, tw, xb, j, odd);
   __syncwarp();
 #pragma unroll
   for (int mc = 0; mc < NC; ++mc)
 #pragma unroll
-    for (int n2 = 0; n2 < T; ++n2) b[mc][n2] = load((j + T * mc) * T + (n2 ^ j));
-  __syncwarp();
+    for (int n2 = 0; n2 < T; ++n2) b[mc][n2] = xb[((j + T * mc) ^ odd) * T + (n2 ^ j)];
+  __syncwarp();   // the places are reused by this group's next transform
 #pragma unroll
   for (int mc = 0; mc < NC; ++mc) {
     float2 X[T];

@@ -131,14 +131,16 @@ __device__ __forceinline__ bool word(uint32_t a, uint32_t b) {
 // (W = 128, L = 4, 1024 positions: two inputs of forty), twenty times what rounding does. So a pass leaves a position with
 // a value within the band (3.9 times that rms) and a jump above kJump of the far fields' norm sqrt(S) W ||p|| to
 // a second launch, which takes the decisions of the whole position from the line transforms, the arithmetic of W = 64:
-// they then depend on the inputs and not on the kernel. At W = 128, L = 4, 1024 positions one pass in five has such a
-// position. Without one the second launch costs 2.2 us (of 672), with one or two 150 us. Deciding within the pass instead
-// was slower throughout: the line transforms' code in this kernel takes registers from all of it (675 -> 715 to 812 us).
+// they then depend on the inputs and not on the kernel. Of the decisions that differ 0.5 % lie outside the band.
+// At W = 128, L = 4, 1024 positions one pass in three has such a position. Without one the second launch costs 2.2 us
+// (of 680), with one or two 155 us; at W = 256, L = 16 1.1 ms (of 44.6). Slower: the decisions within the pass (the line
+// transforms' code takes registers from all of it: 675 -> 715 to 812 us); every position run to its end there and only the
+// difference of the residuals run again (the pass itself 680 -> 686 to 705 us, 65 us saved where no decision differs).
 //
 // Which of this thread's far-field values count as nonzero by that arithmetic: bit 2 k + e for value k of column
-// kc + CH e (wave_kernel's pass C).  The forward model once more, every line by a group of 8 (W = 128) or 16 threads
-// that exchanges through the line's own places, the wave in `sm` (W W / RANKS values per CTA).  Called by every
-// thread of the CTA (cluster), when nothing else needs `sm`; it is free again on return.
+// kc + CH e (wave_kernel's pass C).  The forward model once more, every line by a group of 8 (W = 128) or 16 threads,
+// the wave in `sm` (W W / RANKS values per CTA), exchanges in the places of the fetched transmissions behind it.  Called by
+// every thread of the CTA (cluster), when nothing else needs these; they are free again on return.
 template <int W>
 __device__ __noinline__ uint32_t counted_by_lines(const float2* __restrict__ probe, const float2* __restrict__ T, size_t plane,
                                                   int Nx, int L, float2* sm, const float2* s_w, const float2* s_h1, float zthr2,
@@ -146,7 +148,9 @@ __device__ __noinline__ uint32_t counted_by_lines(const float2* __restrict__ pro
   constexpr int RANKS = W == 256 ? 4 : 1, RW = W / RANKS;          // lines per CTA and direction
   constexpr int TL = W == 128 ? 8 : 16, N1 = W / TL, GROUPS = NT / TL;
   constexpr int RH = W == 128 ? 8 : 4, CH = W / CL;
-  const int j = threadIdx.x % TL, grp = threadIdx.x / TL;
+  const int j = threadIdx.x % TL, grp = threadIdx.x / TL, odd = W == 128 ? grp & 1 : 0;
+  float2* const xb = sm + RC * REGION + grp * W;
+  static_assert(GROUPS * W <= TBUF * NT, "the groups' exchanges fit");
   RegisterTwiddles<W, TL> tw;
 #pragma unroll
   for (int k = 1; k < 8; ++k) tw.r[k] = s_w[k * j];
@@ -172,8 +176,6 @@ __device__ __noinline__ uint32_t counted_by_lines(const float2* __restrict__ pro
 #pragma unroll 1
     for (int r = rank * RW + grp; r < (rank + 1) * RW; r += GROUPS) {
       float2 v[N1], t[N1];
-      auto get = [&](int e) { return sm[at(r, e)]; };
-      auto put = [&](int e, float2 x) { sm[at(r, e)] = x; };
       const float2* Tr = T + l * plane + (size_t)r * Nx + j;
 #pragma unroll
       for (int m = 0; m < N1; ++m) t[m] = Tr[TL * m];   // in flight during the transform
@@ -182,35 +184,33 @@ __device__ __noinline__ uint32_t counted_by_lines(const float2* __restrict__ pro
         for (int m = 0; m < N1; ++m) v[m] = probe[r * W + j + TL * m];
       } else {
 #pragma unroll
-        for (int m = 0; m < N1; ++m) v[m] = get(j + TL * m);
-        line_fft_in_place<W, TL, true>(v, tw, get, put, j);
+        for (int m = 0; m < N1; ++m) v[m] = sm[at(r, j + TL * m)];
+        line_fft_permuted<W, TL, true>(v, tw, xb, j, odd);
       }
 #pragma unroll
       for (int m = 0; m < N1; ++m) v[m] = cmul(v[m], t[m]);
-      line_fft_in_place<W, TL, false>(v, tw, get, put, j);
+      line_fft_permuted<W, TL, false>(v, tw, xb, j, odd);
 #pragma unroll
-      for (int m = 0; m < N1; ++m) put(j + TL * m, v[m]);
+      for (int m = 0; m < N1; ++m) sm[at(r, j + TL * m)] = v[m];
     }
     sync();
 #pragma unroll 1
     for (int c = rank * RW + grp; c < (rank + 1) * RW; c += GROUPS) {
       float2 v[N1];
-      auto get = [&](int e) { return load(e, c); };
-      auto put = [&](int e, float2 x) { store(e, c, x); };
 #pragma unroll
-      for (int m = 0; m < N1; ++m) v[m] = get(j + TL * m);
-      line_fft_in_place<W, TL, false>(v, tw, get, put, j);
+      for (int m = 0; m < N1; ++m) v[m] = load(j + TL * m, c);
+      line_fft_permuted<W, TL, false>(v, tw, xb, j, odd);
       if (l < L - 1) {
         const float2 hx = s_h1[c];
 #pragma unroll
         for (int m = 0; m < N1; ++m) v[m] = cmul(v[m], cmul(s_h1[j + TL * m], hx));
-        line_fft_in_place<W, TL, true>(v, tw, get, put, j);
+        line_fft_permuted<W, TL, true>(v, tw, xb, j, odd);
       } else {
 #pragma unroll
         for (int m = 0; m < N1; ++m) v[m].x = fmaf(v[m].x, v[m].x, v[m].y * v[m].y);
       }
 #pragma unroll
-      for (int m = 0; m < N1; ++m) put(j + TL * m, v[m]);
+      for (int m = 0; m < N1; ++m) store(j + TL * m, c, v[m]);
     }
     sync();
   }

@@ -61,11 +61,11 @@ class Problem:
         self.norm = float(np.sqrt(np.sum(np.abs(self.probe.astype(np.complex128)) ** 2)))
         self.counts = np.full((win, win), np.float32((0.01 * self.norm) ** 2))
 
-    def run(self, msp, call, windows, counts, **kw):
-        """call(g, probe, T, pos, I) with one window and one constant pattern (0 or `counts`) per position."""
+    def run(self, msp, call, windows, counts, where=1.0, **kw):
+        """call(g, probe, T, pos, I) with one window and one pattern (0 or `counts`, at the pixels `where`) per position."""
         cu = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
         g = msp.geometry(**{**self.gd, "n_pos": len(windows)}, param=msp.MSP_PARAM_TRANSMISSION)
-        I = torch.from_numpy(self.counts).cuda()[None] * torch.tensor(counts, dtype=torch.float32, device="cuda")[:, None, None]
+        I = cu((self.counts * where).astype(np.float32))[None] * torch.tensor(counts, dtype=torch.float32, device="cuda")[:, None, None]
         T, p = cu(self.T), cu(self.probe)
         out = call(g, p, T, cu(np.asarray(windows, np.int32)), I.contiguous(), **kw)
         return out, T, p
@@ -75,16 +75,16 @@ class Problem:
         incident, _, psi = O.position_forward(wave, self.T.astype(np.complex128), *at, h)
         return incident, psi, h
 
-    def decisions(self, msp, at):
-        """(bits of the values near the threshold, the gradients of one position, R by them)."""
-        (loss, dT, dp), _, _ = self.run(msp, msp.loss_grad, [at], [1.0])
+    def decisions(self, msp, at, where=1.0):
+        """(bits of the values near the threshold, R, the object's gradient, which pixels these are)."""
+        (loss, dT, dp), _, _ = self.run(msp, msp.loss_grad, [at], [1.0], where)
         dp = dp.cpu().numpy().astype(np.complex128)
         _, psi, _ = self.far_field(self.probe.astype(np.complex128), at)
         R = self.far_field(dp, at)[1] / self.gd["win"] ** 2
         off = np.abs(np.abs(psi) / (O.zero_threshold(self.probe.astype(np.complex128))) - 1.0)
         near = off <= 0.03 * np.sqrt(self.gd["n_slices"])
         counted = np.abs(R - psi) > 0.5 * np.sqrt(self.counts)
-        return counted[near].astype(int), R, dT.cpu().numpy(), dp
+        return counted[near].astype(int), R, dT.cpu().numpy(), near
 
 
 @pytest.mark.parametrize("win,L", CASES)
@@ -93,7 +93,7 @@ def test_values_at_the_threshold_are_decided_as_by_the_line_transforms(msp, win,
     with open(GOLDEN) as f:
         golden = json.load(f)
     for at in ((0, 0), (4, 9)):
-        bits, R, dT, _ = q.decisions(msp, at)
+        bits, R, dT, near = q.decisions(msp, at)
         want = golden[f"{win}_{L}_{at[0]}_{at[1]}"]
         assert len(bits) == len(want) and int((bits != [int(b) for b in want]).sum()) == 0
         # and the object's gradient is that of the same residual
@@ -101,6 +101,12 @@ def test_values_at_the_threshold_are_decided_as_by_the_line_transforms(msp, win,
         grads, _ = O.position_backward(q.T.astype(np.complex128), *at, h, incident, O.dft2_adjoint(R), 0)
         for l, g in grads.items():
             assert rel(dT[l][at[0]:at[0] + win, at[1]:at[1] + win], g) < TOL
+        # a few counts only: the pass lists these values one by one
+        want = np.array([int(b) for b in want])
+        for part in range(12):
+            some = (np.arange(win * win).reshape(win, win) % 89 == 7 * part).astype(np.float32)
+            got = q.decisions(msp, at, some)[0]
+            assert (got == want * some[near]).all()
 
 
 @pytest.mark.parametrize("reduce", [False, True])
