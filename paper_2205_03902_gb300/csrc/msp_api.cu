@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(256) sum_blocks_kernel(const float* __restrict
 // dprobe[i] = sum_b part[b][i], fixed order.  A block of 256 threads owns 32 consecutive probe values: warp g
 // sums the partials b = g, g + 8, g + 16, ... (lane = value, so every load is 256 contiguous bytes), all of
 // them in flight at once, and the eight warp sums are added in warp order.  512 blocks for W = 128 keep
-// every SM loading.  The sums are FP64's to the bit, in compensated FP32: FP64 additions and conversions at 1/64 of the
+// every SM loading.  The sums are as accurate as FP64's, in compensated FP32: FP64 additions and conversions at 1/64 of the
 // FP32 rate took most of the time (64 partials of W = 64: 10.7 us).
 constexpr int kDprobeVals = 32;
 // the sum of value blk kDprobeVals + lane, in the lanes of warp 0

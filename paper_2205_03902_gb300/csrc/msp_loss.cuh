@@ -13,7 +13,7 @@ namespace learn {
 // One thread per pixel: its 16 channels are four 16-byte loads and two 16-byte stores, the target's planes are read in
 // rows.  A thread sums its squares in compensated FP32, rounding errors of the products included, and a pixel whose
 // sum leaves the range where these are exact to FP64's rounding again in FP64: in FP64 alone, whose pipe takes about one
-// conversion or addition per cycle and SM, the kernel took 19 us at 384 x 384 with either split; it takes 9.5.
+// conversion or addition per cycle and SM, the kernel took 19 us at 384 x 384 with either split; it takes 11.
 __global__ void __launch_bounds__(256) loss_kernel(const float* __restrict__ pre, const float* __restrict__ target, int L,
                                                    size_t P, float inv_sd, __nv_bfloat16* __restrict__ g,
                                                    double* __restrict__ part) {

@@ -691,7 +691,7 @@ __global__ void __launch_bounds__(LinesCfg<float2, W>::THREADS) rows_adjoint_ker
 
 // dp64[k] += sum_{b < nb} contrib[b][k], b ascending (fixed order), eight loads in flight per thread.  The sum over
 // a batch is compensated FP32 of FP64's accuracy, added to the FP64 sum once: FP64 additions and conversions of
-// every term took 56 us for 169 positions of W = 128.  Blocks of 64 threads spread the image over the SMs.
+// every term took 83 us for 169 positions of W = 128, this 59.  Blocks of 64 threads spread the image over the SMs.
 __global__ void __launch_bounds__(64) dprobe_accumulate_kernel(const float2* __restrict__ contrib, int nb, int WW,
                                                                double2* __restrict__ dp64, int first) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;

@@ -728,7 +728,7 @@ __global__ void combine_kernel(float2* __restrict__ A, const float2* __restrict_
 //   g_l[k]: slice 0 from g0, slices 1..M-1 summed over the CTAs' partials in a fixed order (32
 //           groups of CTAs, cta mod 32, then the groups in order), in compensated FP32: the FP64
 //           pipe converts and adds about one element per cycle and SM, and the 2 M of them at
-//           N = 40 made this kernel 23 us (26 us with the chain a quarter as long); 9.5 us so;
+//           N = 40 made this kernel 23 us (26 us with the chain a quarter as long); 11 us so;
 //   x = o_l[k] - mu_l lambda g_l[k] in FP64, mu_l = 1 / (lambda prod_{m != l} max|o_m|)^2,
 //       written over o_l[k];
 //   normpart[block] = sum of |x|^2 over the block's 32 elements (fixed order).
